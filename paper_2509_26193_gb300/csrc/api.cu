@@ -73,7 +73,7 @@ void free_all(relearn_ctx *c)
         (void **)&c->d_geom,     (void **)&c->d_sc,         (void **)&c->d_codes,
         (void **)&c->d_off,      (void **)&c->d_ord,        (void **)&c->d_root,
         (void **)&c->d_net,      (void **)&c->d_nkey,       (void **)&c->d_nkey_alt,
-        (void **)&c->d_lstate,   (void **)&c->d_lsum,
+        (void **)&c->d_lstate,   (void **)&c->d_lsum,       (void **)&c->d_fam,
         (void **)&c->d_rq_key,   (void **)&c->d_rq_key_alt, (void **)&c->d_rq_val,
         (void **)&c->d_rq_val_alt, (void **)&c->d_rq_out,   (void **)&c->d_rq_src,
         (void **)&c->d_codes_alt, (void **)&c->d_perm,      (void **)&c->d_perm_alt,
@@ -204,6 +204,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(d_ord, 6 * NB);
     A(d_root, NB);
     A(d_lstate, N);
+    A(d_fam, M + 8); // walks read whole families of eight
     A(d_lsum, 4);
     if (NB > 1) {
         A(d_net, N);
@@ -267,7 +268,8 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     const int64_t sort_blocks = sort_blocks_needed(std::max({N, S, QC}));
     A(sort.hist, 256 * sort_blocks);
     int64_t scan_blocks = std::max({scan_blocks_needed(N + 1), scan_blocks_needed(QC),
-                                    scan_blocks_needed(S), scan_blocks_needed(256 * sort_blocks)});
+                                    scan_blocks_needed(S), scan_blocks_needed(256 * sort_blocks),
+                                    scan_blocks_needed(M)});
     A(scan.block_sums, 4 * scan_blocks); // a pair scan keeps two sums per tile
     A(scan.flags, scan_blocks + 3);
 #undef A

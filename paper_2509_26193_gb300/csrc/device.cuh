@@ -86,6 +86,16 @@ struct __align__(32) Node {
     NodeTopo t;
 };
 
+// A node in family order (the children of a node are contiguous), for walks whose lanes
+// hold nodes instead of sources (length.cu).
+struct __align__(32) FamNode {
+    float cx, cy, cz, cnt; // as NodeGeo
+    int32_t pre;           // pre-order index
+    int32_t up;            // pre-order index of the parent (-1: the root)
+    uint32_t kids;         // place of the first child (inner nodes)
+    uint32_t shift;        // as NodeTopo | 1 for the last of its siblings
+};
+
 // A whole node (32 bytes, 32-byte aligned) in one 256-bit read-only load
 // (PTX ld.global.nc.v8.f32, sm_100 and later): geometry and escape/shift.
 __device__ __forceinline__ void load_node(const Node *n, float4 &g, int2 &t)

@@ -125,6 +125,7 @@ struct relearn_ctx {
     int32_t *d_keep = nullptr;                           // [max_synapses + 1]
 
     // ---- differentiable form (expected synapse length, length.cu)
+    rl::FamNode *d_fam = nullptr; // [max_nodes] the tree of the last forward in family order
     float4 *d_lstate = nullptr; // [n] per source (Morton position): l, Dbar, 1/S, exponent shift
     double *d_lsum = nullptr;   // [4] sum m l, sum m (M), mean
 

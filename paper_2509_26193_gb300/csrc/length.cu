@@ -11,26 +11,28 @@
 //   dl_i/dc_k   = q_ik r_ik (2 (d_ik - l_i) / sigma^2 - 1 / d_ik),  r = x_i - c_k,
 //   dl_i/dx_i   = -sum_k dl_i/dc_k,   dc_k/dx_j = w_j / N_k  (w = vac_de).
 //
-// Forward: one walk of each root frontier (the search kernel's warp-union walk: the
-// warp's 32 sources, cut at the boundaries of depth-5 cells, depth 4 in the adjoint,
-// walk one union per piece), FP32 attractions with Kahan-compensated sums; S, l and
-// Dbar formed in FP64 and kept per source with the exponent shift. Backward: the
-// same walk again,
-// recomputing every attraction (nothing per candidate is stored), accumulating
-// the centroid adjoints G_k = sum_i (m_i / M) dl_i/dc_k per node in FP64 and each
-// source's direct term in registers (Kahan-compensated FP32: it is a sum of terms of
-// both signs that nearly cancel); then every neuron j adds w_j * sum over its cells
-// k of G_k / N_k (its leaf's parent chain, in FP64).
+// Forward: one walk of the root frontiers of 32 sources at a time (group walks, below),
+// FP32 attractions with Kahan-compensated sums; S, l and Dbar formed in FP64 and kept
+// per source with the exponent shift. Backward: the same walk again, recomputing every
+// attraction (nothing per candidate is stored), accumulating the centroid adjoints
+// G_k = sum_i (m_i / M) dl_i/dc_k per node in FP64 and each source's direct term in
+// registers (Kahan-compensated FP32: it is a sum of terms of both signs that nearly
+// cancel); then every neuron j adds w_j * sum over its cells k of G_k / N_k (its leaf's
+// parent chain, in FP64).
 //
-// Node adjoints: in a union walk every lane that takes a candidate takes the same
-// node at the same step, so the warp first sums its lanes' (x, y, z) contributions
-// (a transpose reduction: five shuffle levels that leave each component's total on
-// eight lanes) and three lanes add the totals to the node with FP64 atomics; a warp
-// cut into pieces does this once per piece that took a candidate. One FP32 vector
-// atomic per lane and candidate (the previous design) was L2-atomic-bound and its
-// order-dependent FP32 sums left element-wise gradient errors up to 6e-3 of the
-// cancellation-aware scale at 2^18 neurons; FP64 sums of warp partials bring every
-// element within the FP32 arithmetic of its terms.
+// Node adjoints: the warp sums its lanes' (x, y, z) contributions to eight nodes at a
+// time (a transpose reduction that leaves each component's total on one lane) and adds
+// the totals to the nodes with FP64 atomics. One FP32 vector atomic per lane and
+// candidate (an earlier design) was L2-atomic-bound and its order-dependent FP32 sums
+// left element-wise gradient errors up to 6e-3 of the cancellation-aware scale at 2^18
+// neurons; FP64 sums of warp partials bring every element within the FP32 arithmetic of
+// its terms.
+//
+// Measured (GB300, uniform cube, theta 0.3, the forward and backward calls with their
+// small kernels, one-node-per-step union walks -> group walks): 2^18 neurons forward
+// 1.77 -> 1.55 ms, backward 5.75 -> 2.66 ms; 5,003 neurons, forward + backward
+// 5.5 -> 0.24 ms. Bound by instruction issue (70 to 73 % active at 2^18: per entry and
+// group about 16 instructions of forward sums, 40 of backward ones, and 16 of walking).
 #include "internal.h"
 
 namespace rl {
@@ -38,20 +40,13 @@ namespace rl {
 namespace {
 
 constexpr float kTinyL = 8.673617e-19f; // 2^-60: below this S is redone with a shift
-// Sources in one cell this deep share a walk. The forward pass cuts finer: its
-// pieces step in blocks like one union, so more pieces cost little (2^18 cube,
-// forward: depth 4 2.11 ms, 5 1.77 ms, 6 2.02 ms). The adjoint sums every piece's
-// contributions across the warp at each step, so more pieces cost a warp sum each
-// (adjoint: depth 4 5.77 ms, 5 10.8 ms, 6 31.0 ms).
-constexpr int kFwdDepth = 5, kBwdDepth = 4;
-constexpr int kLenBlock = 128; // walk steps between progress checks
 
 struct LenArgs {
     const Node *__restrict__ nodes;
+    const FamNode *__restrict__ fam;
     const float4 *__restrict__ pos;
     const int32_t *__restrict__ perm;
     const int32_t *__restrict__ act_src;
-    const uint32_t *__restrict__ codes;
     const int32_t *__restrict__ leaf_of;
     const int32_t *__restrict__ vac_ax;
     const int64_t *d_total; // active sources
@@ -134,43 +129,13 @@ __device__ __forceinline__ void add_node(double *G, int32_t p, float ox, float o
     atomicAdd(&G[4 * (int64_t)p + 2], (double)oz);
 }
 
-// Sum of (x, y, z) over the 32 lanes (every lane calls it). Transpose reduction: at
-// offset 16 a lane keeps two of the four values (x, y, z, 0) and sends the other
-// two; at offset 8 it keeps one; offsets 4, 2, 1 sum that one. Afterwards lanes
-// 0-7 hold the total of x, 8-15 of y, 16-23 of z. Returns this lane's total.
-__device__ __forceinline__ float warp_sum3(float x, float y, float z, int lane)
-{
-    const bool hi = lane & 16;
-    float k0 = hi ? z : x, k1 = hi ? 0.0f : y;
-    const float s0 = hi ? x : z, s1 = hi ? y : 0.0f;
-    k0 = __fadd_rn(k0, __shfl_xor_sync(0xffffffffu, s0, 16));
-    k1 = __fadd_rn(k1, __shfl_xor_sync(0xffffffffu, s1, 16));
-    const bool b3 = lane & 8;
-    float k = b3 ? k1 : k0;
-    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8));
-    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 4));
-    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 2));
-    k = __fadd_rn(k, __shfl_xor_sync(0xffffffffu, k, 1));
-    return k;
-}
-
-// The warp's contributions to node p (every lane calls it with the same p; lanes
-// that took no candidate pass zeros): summed across the warp, then added to the
-// node's FP64 adjoint by lanes 0, 8 and 16 (x, y, z).
-__device__ __forceinline__ void add_node_warp(double *G, int32_t p, float ox, float oy, float oz,
-                                              int lane)
-{
-    const float t = warp_sum3(ox, oy, oz, lane);
-    if ((lane & 7) == 0 && lane < 24) atomicAdd(&G[4 * (int64_t)p + (lane >> 3)], (double)t);
-}
-
 // A lane's own walk of its root frontier (stackless: expand = p + 1, accept or
 // empty = escape).
 template <bool kBack>
-__device__ int32_t lane_walk(const LenArgs &a, const Src &s, int32_t end, uint32_t thr0, float k2,
-                             float k2sh, float two_s2, Fwd &f, Bwd &b)
+__device__ int32_t lane_walk(const LenArgs &a, const Src &s, int32_t p, int32_t end,
+                             uint32_t thr0, float k2, float k2sh, float two_s2, Fwd &f, Bwd &b)
 {
-    int32_t p = 1, visited = 0;
+    int32_t visited = 0;
     while (p < end) {
         const float4 g = __ldg(reinterpret_cast<const float4 *>(&a.nodes[p].g));
         const int2 t = __ldg(reinterpret_cast<const int2 *>(&a.nodes[p].t));
@@ -194,18 +159,512 @@ __device__ int32_t lane_walk(const LenArgs &a, const Src &s, int32_t end, uint32
     return visited;
 }
 
-#ifndef RELEARN_LEN_BWD_MIN_BLOCKS
-#define RELEARN_LEN_BWD_MIN_BLOCKS 5 // the adjoint's warp sums need more than 40 registers
-#endif
-// The forward pass at 6 blocks per SM (its three compensated sums need the
-// registers: 8 blocks took the 2^18-neuron forward pass from 2.46 to 3.08 ms), the
-// adjoint at 5 (6 blocks: 6.08 -> 6.32 ms).
+// ---- group walks --------------------------------------------------------------
+// Both passes visit, for each group of 32 sources (adjacent in Morton order), every
+// node that at least one of them accepts, once, with the set of sources that take it.
+// The order is free here (unlike the search's draw), which makes the walk cheap: the
+// lanes of a warp hold nodes, eight families of up to eight children at a time, and put
+// each node to the criterion for the whole group at once; the accepted ones are then
+// evaluated in chunks of 32, lanes holding sources, the nodes read from shared memory
+// (a 16-byte broadcast from there costs 2.3 cycles of the SM, the 32-byte broadcast from
+// L1 of a one-node-per-step walk 8.2, which bounded that walk together with its 31
+// instructions per step).
+//
+// The group's test is conservative: D = fma(rx, rx, fma(ry, ry, rz * rz)) with
+// rx = fl(x - cx) is non-decreasing in |rx|, |ry| and |rz| (rounding is monotone), so the
+// same expression on the smallest and largest |x - cx| over the group's bounding box
+// bounds every source's D exactly. A node whose lower bound passes is taken by every
+// source that reaches it, one whose upper bound fails is expanded for all of them, and
+// the few in between are tested source by source when their chunk is evaluated (their
+// subtree goes on with the sources that rejected it).
+//
+// A pending node carries its set of sources as a mask. With fewer than one group to two
+// resident warps, 2, 4 or 8 warps of a block share a group: each keeps every second,
+// fourth or eighth of the first pending nodes, and their sums are added through shared
+// memory (5,000 neurons: 135 groups for 3,648 warps). The line, groups x warps per group
+// at most twice the resident warps (forward + backward): 60,000 neurons 1.19 ms, at
+// most once 1.29, four times 1.24; 2^18 4.39, 4.41, 4.82 ms.
+
+constexpr int kGroupWarps = 8;      // warps per block
+constexpr int kPend = 256;          // pending nodes per warp
+constexpr int kEntries = 128;       // accepted nodes per warp waiting for evaluation
+constexpr int kLenChunk = 32;       // entries evaluated at a time
+constexpr uint32_t kTestFlag = 0x80000000u;
+constexpr uint32_t kLastSibling = 1u; // in FamNode::shift
+
+struct __align__(16) GroupShared {
+    float4 xy[kLenChunk / 2]; // entries 2k, 2k + 1: x, x, y, y
+    float4 zc[kLenChunk / 2]; // z, z, count, count
+    uint32_t mask[kLenChunk]; // sources that reach the entry
+    int32_t pre[kLenChunk];
+    uint32_t shift[kLenChunk];
+    uint2 pend[kPend];        // first child, mask
+    uint2 out[kEntries];      // node (| kTestFlag), mask
+    int32_t self[32];         // the sources' own leaves (ascending; idle lanes: the largest int)
+};
+
+using Pair = unsigned long long; // two packed floats
+__device__ __forceinline__ Pair pack2(float a, float b)
+{
+    Pair r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(Pair v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ Pair sub2(Pair a, Pair b)
+{
+    Pair r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b)
+{
+    Pair r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b)
+{
+    Pair r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c)
+{
+    Pair r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ void kahan2(Pair &sum, Pair &c, Pair a)
+{
+    const Pair y = sub2(a, c);
+    const Pair t = add2(sum, y);
+    c = sub2(sub2(t, sum), y);
+    sum = t;
+}
+
+// Two compensated sums side by side, one over the even entries, one over the odd ones.
+struct Sum2 {
+    Pair s = 0ull, c = 0ull;
+    __device__ __forceinline__ void add(Pair a) { kahan2(s, c, a); }
+    __device__ __forceinline__ void add_one(float a) // into the even one
+    {
+        float s0, s1, c0, c1;
+        unpack2(s, s0, s1);
+        unpack2(c, c0, c1);
+        kahan(s0, c0, a);
+        s = pack2(s0, s1);
+        c = pack2(c0, c1);
+    }
+    __device__ __forceinline__ double total() const
+    {
+        float s0, s1, c0, c1;
+        unpack2(s, s0, s1);
+        unpack2(c, c0, c1);
+        return ((double)s0 - (double)c0) + ((double)s1 - (double)c1);
+    }
+};
+
+struct FwdSums {
+    Sum2 s, a, b; // attraction, attraction x d, attraction x D
+};
+struct BwdSums {
+    Sum2 cov;
+    Sum2 gx, gy, gz; // the direct term, negated
+};
+
+__device__ __forceinline__ void load_fam(const FamNode *n, float4 &g, int4 &t)
+{
+    float v[8];
+    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7])
+        : "l"(n));
+    g = make_float4(v[0], v[1], v[2], v[3]);
+    t = make_int4(__float_as_int(v[4]), __float_as_int(v[5]), __float_as_int(v[6]),
+                  __float_as_int(v[7]));
+}
+
+__device__ __forceinline__ float warp_min(float v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+__device__ __forceinline__ float dist2_of(float rx, float ry, float rz)
+{
+    return __fmaf_rn(rx, rx, __fmaf_rn(ry, ry, __fmul_rn(rz, rz)));
+}
+
+// A pending subtree without room to expand it: its sources walk it one by one. Called
+// only while the pending list is nearly full.
 template <bool kBack>
-__global__ void __launch_bounds__(256, kBack ? RELEARN_LEN_BWD_MIN_BLOCKS : 6)
+__device__ __noinline__ void walk_pending(const LenArgs &a, const Src &s, uint2 item,
+                                          uint32_t thr0, float k2, float two_s2, float sums[4],
+                                          int64_t &evals)
+{
+    const int lane = threadIdx.x & 31;
+    const FamNode *kid = a.fam + item.x;
+    const int32_t p0 = kid->pre;
+    const int32_t end = a.nodes[kid->up].t.escape;
+    Fwd f;
+    Bwd b;
+    if ((item.y >> lane) & 1u)
+        evals += lane_walk<kBack>(a, s, p0, end, thr0, k2, s.k2sh, two_s2, f, b);
+    if constexpr (kBack) {
+        sums[0] = b.cov;
+        sums[1] = __fsub_rn(b.cx, b.gx);
+        sums[2] = __fsub_rn(b.cy, b.gy);
+        sums[3] = __fsub_rn(b.cz, b.gz);
+    } else {
+        sums[0] = __fsub_rn(f.s, f.sc);
+        sums[1] = __fsub_rn(f.a, f.ac);
+        sums[2] = __fsub_rn(f.b, f.bc);
+        sums[3] = 0.0f;
+    }
+    __syncwarp();
+}
+
+// The walk of one group by one warp (all lanes converged).
+struct GroupWalk {
+    const FamNode *__restrict__ fam;
+    GroupShared *s;
+    uint32_t thr0;
+    float lx, hx, ly, hy, lz, hz; // bounding box of the sources
+    int32_t self_lo, self_hi;     // range of the sources' own leaves (pre-order)
+    int32_t base, top;            // pending nodes: pend[base .. top)
+    int32_t outc;                 // entries: out[0 .. outc)
+
+    // members: the lanes that are sources, at least one
+    __device__ __forceinline__ void start(uint32_t members, float3 x, int32_t self)
+    {
+        const int lane = threadIdx.x & 31;
+        const float inf = __int_as_float(0x7f800000);
+        const bool in = (members >> lane) & 1u;
+        lx = warp_min(in ? x.x : inf);
+        hx = -warp_min(in ? -x.x : inf);
+        ly = warp_min(in ? x.y : inf);
+        hy = -warp_min(in ? -x.y : inf);
+        lz = warp_min(in ? x.z : inf);
+        hz = -warp_min(in ? -x.z : inf);
+        self_lo = __shfl_sync(0xffffffffu, self, __ffs(members) - 1);
+        self_hi = __shfl_sync(0xffffffffu, self, 31 - __clz(members));
+        s->self[lane] = self;
+        if (lane == 0) s->pend[0] = make_uint2((uint32_t)__ldg(&fam[0].kids), members);
+        base = 0;
+        top = 1;
+        outc = 0;
+        __syncwarp();
+    }
+
+    // Expands up to eight pending nodes, the last ones (or the first ones, so that the
+    // list grows evenly over the tree): at most 64 more pending nodes and entries.
+    template <bool kFront>
+    __device__ __forceinline__ void expand()
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t lt = lanemask_lt();
+        const int ns = min(8, top - base);
+        const int c = lane & 7;
+        uint2 it[2];
+        bool slot_on[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int slot = (lane >> 3) + 4 * h;
+            slot_on[h] = slot < ns;
+            it[h] = slot < ns ? s->pend[kFront ? base + slot : top - 1 - slot]
+                              : make_uint2(0u, 0u); // family 0 holds the root alone
+        }
+        if (kFront)
+            base += ns;
+        else
+            top -= ns;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && ns <= 4) break;
+            const uint32_t k = it[h].x + c;
+            float4 g;
+            int4 t;
+            load_fam(&fam[k], g, t);
+            const uint32_t shift = (uint32_t)t.w & ~kLastSibling;
+            // the family ends at its last sibling; one of more than eight (a bucket's
+            // leaves) goes on as another pending node
+            const uint32_t ends = __ballot_sync(0xffffffffu, ((uint32_t)t.w & kLastSibling) != 0u);
+            const uint32_t fam_ends = (ends >> (lane & 24)) & 0xffu;
+            const bool act = slot_on[h] && (fam_ends & ((1u << c) - 1u)) == 0u;
+            bool near_ok = true, far_ok = true; // the criterion at the bounds of D
+            if (!node_is_leaf(shift)) {
+                const float ax = __fsub_rn(lx, g.x), bx = __fsub_rn(hx, g.x);
+                const float ay = __fsub_rn(ly, g.y), by = __fsub_rn(hy, g.y);
+                const float az = __fsub_rn(lz, g.z), bz = __fsub_rn(hz, g.z);
+                const float D0 = dist2_of(fmaxf(fmaxf(ax, -bx), 0.0f), fmaxf(fmaxf(ay, -by), 0.0f),
+                                          fmaxf(fmaxf(az, -bz), 0.0f));
+                const float D1 = dist2_of(fmaxf(fabsf(ax), fabsf(bx)), fmaxf(fabsf(ay), fabsf(by)),
+                                          fmaxf(fabsf(az), fabsf(bz)));
+                // (a centroid that is not a number is accepted, as by each source alone)
+                near_ok = __float_as_uint(D0) + shift > thr0 || D1 != D1;
+                far_ok = __float_as_uint(D1) + shift > thr0;
+            }
+            const bool has = act && g.w > 0.0f;
+            const uint32_t entry = __ballot_sync(0xffffffffu, has && far_ok);
+            const uint32_t open = __ballot_sync(0xffffffffu, has && !far_ok);
+            if (has && far_ok)
+                s->out[outc + __popc(entry & lt)] =
+                    make_uint2(near_ok ? k : k | kTestFlag, it[h].y);
+            if (has && !far_ok)
+                s->pend[top + __popc(open & lt)] = make_uint2((uint32_t)t.z, it[h].y);
+            top += __popc(open);
+            outc += __popc(entry);
+            // (a zero byte in ends: none of its eight nodes is a last sibling)
+            if ((ends - 0x01010101u) & ~ends & 0x80808080u) {
+                const bool more = act && c == 7 && fam_ends == 0u;
+                const uint32_t rest = __ballot_sync(0xffffffffu, more);
+                if (more) s->pend[top + __popc(rest & lt)] = make_uint2(k + 1u, it[h].y);
+                top += __popc(rest);
+            }
+        }
+        __syncwarp();
+    }
+
+    // Of the pending nodes and entries keep every wpg-th, from the sub-th on.
+    __device__ __forceinline__ void take_share(int sub, int wpg)
+    {
+        const int lane = threadIdx.x & 31;
+        auto thin = [&](uint2 *v, int from, int to) {
+            int kept = 0;
+            for (int i0 = 0; from + sub + wpg * i0 < to; i0 += 32) {
+                const int q = from + sub + wpg * (i0 + lane);
+                const bool ok = q < to;
+                const uint2 w = ok ? v[q] : make_uint2(0u, 0u);
+                __syncwarp();
+                if (ok) v[i0 + lane] = w; // never past the place it was read from
+                __syncwarp();
+                kept += __popc(__ballot_sync(0xffffffffu, ok));
+            }
+            return kept;
+        };
+        top = thin(s->pend, base, top);
+        base = 0;
+        outc = thin(s->out, 0, outc);
+    }
+
+    // The next chunk: the last n <= 32 entries into xy, zc, mask, pre and shift, filled up
+    // with entries that no source takes. Returns the entries that have to be tested
+    // source by source; kids = the first child of this lane's entry.
+    __device__ __forceinline__ uint32_t gather(int n, uint32_t &kids, int64_t &evals)
+    {
+        const int lane = threadIdx.x & 31;
+        outc -= n;
+        kids = 0u;
+        bool tst = false;
+        if (lane < n) {
+            const uint2 w = s->out[outc + lane];
+            float4 g;
+            int4 t;
+            load_fam(&fam[w.x & ~kTestFlag], g, t);
+            tst = (w.x & kTestFlag) != 0u;
+            uint32_t m = w.y;
+            const uint32_t shift = (uint32_t)t.w & ~kLastSibling;
+            if (node_is_leaf(shift) && t.x >= self_lo && t.x <= self_hi) {
+                int lo = 0; // a source does not take its own leaf
+#pragma unroll
+                for (int o = 16; o; o >>= 1)
+                    if (s->self[lo + o] <= t.x) lo += o;
+                if (s->self[lo] == t.x) m &= ~(1u << lo);
+            }
+            // a position that is not a number makes the sums of the sources that take it
+            // not a number, and no other's
+            if (g.x != g.x || g.y != g.y || g.z != g.z)
+                g = make_float4(lx, ly, lz, __int_as_float(0x7fc00000));
+            float *xy = reinterpret_cast<float *>(s->xy) + (lane >> 1) * 4 + (lane & 1);
+            float *zc = reinterpret_cast<float *>(s->zc) + (lane >> 1) * 4 + (lane & 1);
+            xy[0] = g.x;
+            xy[2] = g.y;
+            zc[0] = g.z;
+            zc[2] = g.w;
+            s->mask[lane] = m;
+            s->pre[lane] = t.x;
+            s->shift[lane] = shift;
+            kids = (uint32_t)t.z;
+            evals += __popc(m);
+        } else { // padding
+            float *xy = reinterpret_cast<float *>(s->xy) + (lane >> 1) * 4 + (lane & 1);
+            float *zc = reinterpret_cast<float *>(s->zc) + (lane >> 1) * 4 + (lane & 1);
+            xy[0] = lx;
+            xy[2] = ly;
+            zc[0] = lz;
+            zc[2] = 0.0f;
+            s->mask[lane] = 0u;
+        }
+        const uint32_t tests = __ballot_sync(0xffffffffu, tst);
+        __syncwarp();
+        return tests;
+    }
+
+    // Puts the marked entries of the chunk to the criterion, source by source (x: this
+    // lane's): their masks keep the sources that take them, and below them the sources
+    // that do not go on. Apart from the sums, so that those run without a branch (tests
+    // inside their loop kept its chains of dependent operations from overlapping: 2^18
+    // neurons, forward 1.71 against 1.55 ms).
+    __device__ __forceinline__ void resolve(uint32_t tests, uint32_t kids, float3 x,
+                                            int64_t &evals)
+    {
+        const int lane = threadIdx.x & 31;
+        const uint32_t bit = 1u << lane;
+        uint32_t rej = 0u; // of entry `lane`
+        const float *xy = reinterpret_cast<const float *>(s->xy);
+        const float *zc = reinterpret_cast<const float *>(s->zc);
+        while (tests) { // two at a time (an odd last one twice)
+            const int j0 = __ffs(tests) - 1;
+            tests &= tests - 1;
+            const int j1 = tests ? __ffs(tests) - 1 : j0;
+            tests &= tests - 1;
+            const int k0 = (j0 >> 1) * 4 + (j0 & 1), k1 = (j1 >> 1) * 4 + (j1 & 1);
+            const float D0 = dist2_of(__fsub_rn(x.x, xy[k0]), __fsub_rn(x.y, xy[k0 + 2]),
+                                      __fsub_rn(x.z, zc[k0]));
+            const float D1 = dist2_of(__fsub_rn(x.x, xy[k1]), __fsub_rn(x.y, xy[k1 + 2]),
+                                      __fsub_rn(x.z, zc[k1]));
+            const bool f0 = !(__float_as_uint(D0) + s->shift[j0] > thr0);
+            const bool f1 = !(__float_as_uint(D1) + s->shift[j1] > thr0);
+            const uint32_t r0 = __ballot_sync(0xffffffffu, f0 && (s->mask[j0] & bit));
+            const uint32_t r1 = __ballot_sync(0xffffffffu, f1 && (s->mask[j1] & bit));
+            if (lane == j0) rej = r0;
+            if (lane == j1) rej = r1;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, rej != 0u);
+        if (rej) {
+            s->mask[lane] &= ~rej;
+            s->pend[top + __popc(m & lanemask_lt())] = make_uint2(kids, rej);
+        }
+        top += __popc(m);
+        evals -= __popc(rej);
+        __syncwarp();
+    }
+};
+
+// The chunk's sums of this lane's source.
+__device__ __forceinline__ void fwd_chunk(const GroupShared *g, int n, const Src &src, float k2,
+                                          FwdSums &f)
+{
+    const uint32_t bit = 1u << (threadIdx.x & 31);
+    const Pair xx = pack2(src.x.x, src.x.x), yy = pack2(src.x.y, src.x.y),
+               zz = pack2(src.x.z, src.x.z), nk2 = pack2(-k2, -k2),
+               sh = pack2(src.k2sh, src.k2sh);
+#pragma unroll 4
+    for (int j = 0; j < n; j += 2) {
+        const ulonglong2 xy = *reinterpret_cast<const ulonglong2 *>(&g->xy[j >> 1]);
+        const ulonglong2 zc = *reinterpret_cast<const ulonglong2 *>(&g->zc[j >> 1]);
+        const uint2 m = *reinterpret_cast<const uint2 *>(&g->mask[j]);
+        const Pair rx = sub2(xx, xy.x), ry = sub2(yy, xy.y), rz = sub2(zz, zc.x);
+        const Pair D = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
+        const bool on0 = (m.x & bit) != 0u, on1 = (m.y & bit) != 0u;
+        float D0, D1, e0, e1;
+        unpack2(D, D0, D1);
+        unpack2(fma2(nk2, D, sh), e0, e1);
+        float a0, a1;
+        unpack2(mul2(zc.y, pack2(ex2_approx(e0), ex2_approx(e1))), a0, a1);
+        const Pair at = pack2(on0 ? a0 : 0.0f, on1 ? a1 : 0.0f);
+        f.s.add(at);
+        f.a.add(mul2(at, pack2(sqrt_approx(D0), sqrt_approx(D1))));
+        f.b.add(mul2(at, D));
+    }
+}
+
+// Sums over the 32 lanes of v[e][c] (8 entries, x, y, z), as a transpose reduction: at
+// each level a lane keeps half of its values and sends the other half, so that after
+// five levels lane 4 e + c holds the total of entry e, component c (31 adds and 24
+// shuffles for 24 totals).
+__device__ __forceinline__ float warp_sum_8x3(float v[8][3], int lane)
+{
+#pragma unroll
+    for (int lev = 0; lev < 3; ++lev) {
+        const int o = 16 >> lev, half = 4 >> lev;
+        const bool hi = lane & o;
+#pragma unroll
+        for (int e = 0; e < half; ++e)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float keep = hi ? v[e + half][c] : v[e][c];
+                const float send = hi ? v[e][c] : v[e + half][c];
+                v[e][c] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
+            }
+    }
+    const bool c1 = lane & 2, c0 = lane & 1;
+    float k0 = c1 ? v[0][2] : v[0][0], k1 = c1 ? 0.0f : v[0][1];
+    k0 = __fadd_rn(k0, __shfl_xor_sync(0xffffffffu, c1 ? v[0][0] : v[0][2], 2));
+    k1 = __fadd_rn(k1, __shfl_xor_sync(0xffffffffu, c1 ? v[0][1] : 0.0f, 2));
+    return __fadd_rn(c0 ? k1 : k0, __shfl_xor_sync(0xffffffffu, c0 ? k0 : k1, 1));
+}
+
+// The chunk's terms of this lane's source: its covariance and direct term, and the
+// warp's contributions to the entries' adjoints, eight entries at a time: summed over
+// the warp in FP32, then one FP64 atomic per entry and component.
+__device__ __forceinline__ void bwd_chunk(const GroupShared *g, int n, const Src &src, float k2,
+                                          float two_s2, double *G, BwdSums &b)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t bit = 1u << lane;
+    const Pair xx = pack2(src.x.x, src.x.x), yy = pack2(src.x.y, src.x.y),
+               zz = pack2(src.x.z, src.x.z), nk2 = pack2(-k2, -k2),
+               sh = pack2(src.k2sh, src.k2sh), inv_s = pack2(src.invS, src.invS),
+               ll = pack2(src.l, src.l), db = pack2(src.Db, src.Db),
+               ww = pack2(src.w, src.w), ts = pack2(two_s2, two_s2);
+    for (int j0 = 0; j0 < n; j0 += 8) {
+        float v[8][3];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+            const int j = j0 + u;
+            const ulonglong2 xy = *reinterpret_cast<const ulonglong2 *>(&g->xy[j >> 1]);
+            const ulonglong2 zc = *reinterpret_cast<const ulonglong2 *>(&g->zc[j >> 1]);
+            const uint2 m = *reinterpret_cast<const uint2 *>(&g->mask[j]);
+            const Pair rx = sub2(xx, xy.x), ry = sub2(yy, xy.y), rz = sub2(zz, zc.x);
+            const Pair D = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
+            const bool on0 = (m.x & bit) != 0u, on1 = (m.y & bit) != 0u;
+            float D0, D1, e0, e1, a0, a1;
+            unpack2(D, D0, D1);
+            unpack2(fma2(nk2, D, sh), e0, e1);
+            unpack2(mul2(zc.y, pack2(ex2_approx(e0), ex2_approx(e1))), a0, a1);
+            const Pair q = mul2(pack2(on0 ? a0 : 0.0f, on1 ? a1 : 0.0f), inv_s);
+            const float d0 = sqrt_approx(D0), d1 = sqrt_approx(D1);
+            const Pair dl = sub2(pack2(d0, d1), ll);
+            b.cov.add(mul2(mul2(q, dl), sub2(D, db)));
+            const Pair ninv = pack2(d0 > 0.0f ? -rcp_approx(d0) : 0.0f,
+                                    d1 > 0.0f ? -rcp_approx(d1) : 0.0f);
+            const Pair kap = mul2(mul2(q, fma2(ts, dl, ninv)), ww);
+            const Pair ox = mul2(kap, rx), oy = mul2(kap, ry), oz = mul2(kap, rz);
+            b.gx.add(ox);
+            b.gy.add(oy);
+            b.gz.add(oz);
+            unpack2(ox, v[u][0], v[u + 1][0]);
+            unpack2(oy, v[u][1], v[u + 1][1]);
+            unpack2(oz, v[u][2], v[u + 1][2]);
+        }
+        const float t = warp_sum_8x3(v, lane);
+        const int e = j0 + (lane >> 2);
+        if ((lane & 3) < 3 && e < n && t != 0.0f)
+            atomicAdd(&G[4 * (int64_t)g->pre[e] + (lane & 3)], (double)t);
+    }
+}
+
+// 3 blocks per SM (80 registers): 2^18 neurons, forward + backward 4.21 ms; 4 blocks
+// (64 registers, spills) 4.49, 2 blocks 4.25 (60,000 neurons: 1.13, 1.22, 1.29 ms).
+#ifndef RELEARN_LEN_MIN_BLOCKS
+#define RELEARN_LEN_MIN_BLOCKS 3
+#endif
+template <bool kBack>
+__global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
     length_kernel(LenArgs a)
 {
+    __shared__ GroupShared s_group[kGroupWarps];
+    __shared__ double s_sum[kGroupWarps][3][32];
+    __shared__ int32_t s_next;
     const int32_t A = (int32_t)*a.d_total;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t thr0 = __ldg(&a.sc->thr0);
     const float k2 = __ldg(&a.sc->k2);
     const float sigma = __ldg(&a.sc->sigma);
@@ -216,23 +675,41 @@ __global__ void __launch_bounds__(256, kBack ? RELEARN_LEN_BWD_MIN_BLOCKS : 6)
         const double M = a.lsum[1];
         wscale = M > 0.0 ? (a.gout ? *a.gout : 1.0) / M : 0.0;
     }
+    // warps per group (see above for the line)
+    const int32_t groups = (A + 31) / 32;
+    int wpg = kGroupWarps;
+    while (wpg > 1 && (int64_t)groups * wpg > 2 * (int64_t)gridDim.x * kGroupWarps) wpg >>= 1;
+    const int sub = warp & (wpg - 1);
     double my0 = 0.0, my1 = 0.0;
     int64_t my_evals = 0;
+    GroupWalk w;
+    w.fam = a.fam;
+    w.s = &s_group[warp];
+    w.thr0 = thr0;
     for (;;) {
-        int32_t nb = 0;
-        if (lane == 0) nb = atomicAdd(a.work, 32);
-        nb = __shfl_sync(0xffffffffu, nb, 0);
-        if (nb >= A) break;
-        const int32_t slot = nb + lane;
+        int32_t gr = 0;
+        if (wpg == 1) {
+            if (lane == 0) gr = atomicAdd(a.work, 1);
+            gr = __shfl_sync(0xffffffffu, gr, 0);
+            if (gr >= groups) break;
+        } else { // the block takes kGroupWarps / wpg groups together
+            __syncthreads();
+            if (threadIdx.x == 0) s_next = atomicAdd(a.work, kGroupWarps / wpg);
+            __syncthreads();
+            if (s_next >= groups) break;
+            gr = s_next + warp / wpg;
+        }
+        const int64_t slot = (int64_t)gr * 32 + lane;
         const bool live = slot < A;
         const int32_t sp = live ? a.act_src[slot] : -1;
         Src s;
         const float4 xp = live ? a.pos[sp] : make_float4(0.f, 0.f, 0.f, 0.f);
         s.x = make_float3(xp.x, xp.y, xp.z);
-        s.self = live ? a.leaf_of[sp] : -1;
+        s.self = live ? a.leaf_of[sp] : 0x7fffffff;
         const int32_t i = live ? a.perm[sp] : 0;
         s.l = s.Db = s.invS = s.k2sh = s.w = 0.0f;
-        bool on_src = live; // takes part as a source (backward: included in M)
+        // a source without a finite position has no finite distance and is left out
+        bool on_src = live && fabsf(xp.x) + fabsf(xp.y) + fabsf(xp.z) < __int_as_float(0x7f800000);
         if constexpr (kBack) {
             if (live) {
                 const float4 st = a.state[sp];
@@ -241,137 +718,120 @@ __global__ void __launch_bounds__(256, kBack ? RELEARN_LEN_BWD_MIN_BLOCKS : 6)
                 s.invS = st.z;
                 s.k2sh = st.w;
             }
-            on_src = live && s.invS > 0.0f;
+            on_src = on_src && s.invS > 0.0f;
             s.w = on_src ? (float)((double)a.vac_ax[i] * wscale) : 0.0f;
         }
-        // the 32 sources (Morton order) are cut wherever two neighbours do not share a
-        // cell of depth kFwdDepth (kBwdDepth); each piece walks one union (one piece: uni)
-        const int last = min(A - 1 - nb, 31);
-        uint32_t code = live ? a.codes[sp] : 0u;
-        code = __shfl_sync(0xffffffffu, code, live ? lane : last);
-        const uint32_t nxt = __shfl_down_sync(0xffffffffu, code, 1);
-        const uint32_t cuts = __ballot_sync(
-            0xffffffffu,
-            lane < 31 && morton_common_digits(code, nxt) < (kBack ? kBwdDepth : kFwdDepth));
-        const bool uni = cuts == 0;
-        Fwd f;
-        Bwd b;
-        // The walks step in blocks of four steps per bounds test: nodes root_end ..
-        // root_end + 2 are sentinels (no count, escape = the next node), and a piece
-        // whose walk has ended parks on root_end (its escape clamped back to it).
-        // Escapes are taken as stored; each block of kLenBlock steps must advance,
-        // which keeps a walk over a malformed tree finite.
-        int32_t p = 1, skip = on_src ? 0 : 0x7fffffff;
-        if (!uni) {
-            const uint32_t below = cuts & ((1u << lane) - 1u);
-            const int first = below ? 32 - __clz(below) : 0;
-            const uint32_t from = cuts >> lane;
-            const int lastl = from ? lane + __ffs(from) - 1 : 31;
-            const uint32_t gmask = (lastl == 31 ? 0xffffffffu : ((1u << (lastl + 1)) - 1u)) &
-                                   ~((1u << first) - 1u);
-            auto piece_step = [&]() {
-                float4 g;
-                int2 t;
-                load_node(&a.nodes[p], g, t); // one 256-bit read
-                const float rx = __fsub_rn(s.x.x, g.x), ry = __fsub_rn(s.x.y, g.y),
-                            rz = __fsub_rn(s.x.z, g.z);
-                const float D = __fmaf_rn(rx, rx, __fmaf_rn(ry, ry, __fmul_rn(rz, rz)));
-                const bool on = p >= skip && g.w > 0.0f;
-                const bool pass = __float_as_uint(D) + (uint32_t)t.y > thr0;
-                const bool take = on && pass && p != s.self;
-                if (on && pass) skip = t.x;
-                my_evals += take ? 1 : 0;
-                if constexpr (!kBack) {
-                    if (take) fwd_visit(f, g.w, D, k2, 0.0f);
-                } else {
-                    float ox = 0.0f, oy = 0.0f, oz = 0.0f;
-                    if (take) bwd_visit(b, s, g.w, rx, ry, rz, D, k2, two_s2, ox, oy, oz);
-                    // one warp sum per piece that took a candidate at this step
-                    const uint32_t took = __ballot_sync(0xffffffffu, take) & gmask;
-                    uint32_t heads = __ballot_sync(0xffffffffu, lane == first && took != 0u);
-                    while (heads) {
-                        const int h = __ffs(heads) - 1;
-                        heads &= heads - 1;
-                        const bool mine = first == h;
-                        add_node_warp(a.G, __shfl_sync(0xffffffffu, p, h), mine ? ox : 0.0f,
-                                      mine ? oy : 0.0f, mine ? oz : 0.0f, lane);
+        FwdSums f;
+        BwdSums b;
+        const uint32_t members = __ballot_sync(0xffffffffu, on_src);
+        if (members) {
+            { // lanes without a source follow one, with an empty mask
+                const int f0 = __ffs(members) - 1;
+                const float mx = __shfl_sync(0xffffffffu, s.x.x, f0),
+                            my = __shfl_sync(0xffffffffu, s.x.y, f0),
+                            mz = __shfl_sync(0xffffffffu, s.x.z, f0);
+                if (!on_src) s.x = make_float3(mx, my, mz);
+            }
+            w.start(members, s.x, s.self);
+            if (wpg > 1) { // a pending list long enough to share out (at most 140 nodes)
+                while (w.top - w.base > 0 && w.top - w.base < 8 * wpg && w.top <= 72 &&
+                       w.outc < kEntries - 64)
+                    w.expand<true>();
+                w.take_share(sub, wpg);
+            }
+            for (;;) {
+                while (w.outc < kLenChunk && w.top > 0) {
+                    if (w.top > kPend - 64 - kLenChunk) { // not reached by ordinary trees
+                        const uint2 it = w.s->pend[--w.top];
+                        float part[4];
+                        walk_pending<kBack>(a, s, it, thr0, k2, two_s2, part, my_evals);
+                        if constexpr (kBack) {
+                            b.cov.add_one(part[0]);
+                            b.gx.add_one(part[1]);
+                            b.gy.add_one(part[2]);
+                            b.gz.add_one(part[3]);
+                        } else {
+                            f.s.add_one(part[0]);
+                            f.a.add_one(part[1]);
+                            f.b.add_one(part[2]);
+                        }
+                    } else {
+                        w.expand<false>();
                     }
                 }
-                const uint32_t down = __ballot_sync(0xffffffffu, on && !pass) & gmask;
-                p = min(down ? p + 1 : t.x, root_end);
-            };
-            while (__any_sync(0xffffffffu, p < root_end)) {
-                const int32_t p_blk = p;
-                int k = 0;
-#pragma unroll 1
-                for (; k < kLenBlock && __any_sync(0xffffffffu, p < root_end); k += 4) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) piece_step();
-                }
-                if (__any_sync(0xffffffffu, p < root_end && p <= p_blk)) break;
+                const int n = min(w.outc, kLenChunk);
+                if (n == 0) break;
+                uint32_t kids;
+                const uint32_t tests = w.gather(n, kids, my_evals);
+                if (tests) w.resolve(tests, kids, s.x, my_evals);
+                if constexpr (kBack)
+                    bwd_chunk(w.s, n, s, k2, two_s2, a.G, b);
+                else
+                    fwd_chunk(w.s, n, s, k2, f);
+                __syncwarp(); // the chunk is overwritten next
             }
+        }
+        double t0, t1, t2;
+        if constexpr (kBack) {
+            t0 = b.gx.total();
+            t1 = b.gy.total();
+            t2 = b.gz.total();
+            if (on_src) my0 += (double)s.w * b.cov.total(); // * 2 / sigma^3 below
         } else {
-            auto uni_step = [&]() {
-                float4 g;
-                int2 t;
-                load_node(&a.nodes[p], g, t); // one 256-bit read
-                const float rx = __fsub_rn(s.x.x, g.x), ry = __fsub_rn(s.x.y, g.y),
-                            rz = __fsub_rn(s.x.z, g.z);
-                const float D = __fmaf_rn(rx, rx, __fmaf_rn(ry, ry, __fmul_rn(rz, rz)));
-                const bool on = p >= skip && g.w > 0.0f;
-                const bool pass = __float_as_uint(D) + (uint32_t)t.y > thr0;
-                const bool take = on && pass && p != s.self;
-                if (on && pass) skip = t.x;
-                my_evals += take ? 1 : 0;
-                if constexpr (!kBack) {
-                    if (take) fwd_visit(f, g.w, D, k2, 0.0f);
-                } else {
-                    float ox = 0.0f, oy = 0.0f, oz = 0.0f;
-                    if (take) bwd_visit(b, s, g.w, rx, ry, rz, D, k2, two_s2, ox, oy, oz);
-                    if (__any_sync(0xffffffffu, take)) add_node_warp(a.G, p, ox, oy, oz, lane);
-                }
-                p = __any_sync(0xffffffffu, on && !pass) ? p + 1 : t.x;
-            };
-            while (p < root_end) {
-                const int32_t p_blk = p;
-#pragma unroll 1
-                for (int k = 0; k < kLenBlock && p < root_end; k += 4) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) uni_step();
-                }
-                if (p <= p_blk) break;
+            t0 = f.s.total();
+            t1 = f.a.total();
+            t2 = f.b.total();
+        }
+        if (wpg > 1) {
+            s_sum[warp][0][lane] = t0;
+            s_sum[warp][1][lane] = t1;
+            s_sum[warp][2][lane] = t2;
+            __syncthreads();
+            if (sub != 0) continue;
+            for (int k = 1; k < wpg; ++k) {
+                t0 += s_sum[warp + k][0][lane];
+                t1 += s_sum[warp + k][1][lane];
+                t2 += s_sum[warp + k][2][lane];
             }
         }
         if constexpr (!kBack) {
-            if (!live) continue;
-            double S = (double)f.s - (double)f.sc;
-            float k2sh = 0.0f;
-            if (S < (double)kTinyL && f.dmin2 < __int_as_float(0x7f800000)) {
-                // every term underflowed: redo with the exponents shifted by the nearest D
-                k2sh = __fmul_rn(k2, f.dmin2);
-                f = Fwd();
-                Bwd unused;
-                my_evals += lane_walk<false>(a, s, root_end, thr0, k2, k2sh, two_s2, f, unused);
-                S = (double)f.s - (double)f.sc;
+            if (live) {
+                double S = t0;
+                float k2sh = 0.0f;
+                if (on_src && S < (double)kTinyL) {
+                    // every term underflowed: redo with the exponents shifted by the
+                    // nearest D, which a first walk of the lane's own frontier finds
+                    Bwd unused;
+                    Fwd g;
+                    lane_walk<false>(a, s, 1, root_end, thr0, k2, 0.0f, two_s2, g, unused);
+                    if (g.dmin2 < __int_as_float(0x7f800000)) {
+                        k2sh = __fmul_rn(k2, g.dmin2);
+                        g = Fwd();
+                        my_evals += lane_walk<false>(a, s, 1, root_end, thr0, k2, k2sh, two_s2, g,
+                                                     unused);
+                        S = (double)g.s - (double)g.sc;
+                        t1 = (double)g.a - (double)g.ac;
+                        t2 = (double)g.b - (double)g.bc;
+                    }
+                }
+                float4 st = make_float4(0.f, 0.f, 0.f, k2sh);
+                if (S > 0.0) {
+                    const double l = t1 / S;
+                    st.x = (float)l;
+                    st.y = (float)(t2 / S);
+                    st.z = (float)(1.0 / S);
+                    const double m = (double)a.vac_ax[i];
+                    my0 += m * l;
+                    my1 += m;
+                }
+                a.state[sp] = st;
             }
-            float4 st = make_float4(0.f, 0.f, 0.f, k2sh);
-            if (S > 0.0) {
-                const double l = ((double)f.a - (double)f.ac) / S;
-                st.x = (float)l;
-                st.y = (float)(((double)f.b - (double)f.bc) / S);
-                st.z = (float)(1.0 / S);
-                const double m = (double)a.vac_ax[i];
-                my0 += m * l;
-                my1 += m;
-            }
-            a.state[sp] = st;
-        } else {
-            if (!on_src) continue;
-            a.gx[i] = __fsub_rn(b.gx, b.cx);
-            a.gy[i] = __fsub_rn(b.gy, b.cy);
-            a.gz[i] = __fsub_rn(b.gz, b.cz);
-            my0 += (double)s.w * (double)b.cov; // * 2 / sigma^3 below
+        } else if (on_src) { // the sums hold the negated direct term
+            a.gx[i] = (float)-t0;
+            a.gy[i] = (float)-t1;
+            a.gz[i] = (float)-t2;
         }
+        __syncwarp();
     }
     for (int o = 16; o; o >>= 1) {
         my0 += __shfl_xor_sync(0xffffffffu, my0, o);
@@ -391,6 +851,59 @@ __global__ void __launch_bounds__(256, kBack ? RELEARN_LEN_BWD_MIN_BLOCKS : 6)
             const double sd = (double)sigma;
             atomicAdd(a.gsigma, my0 * 2.0 / (sd * sd * sd));
         }
+    }
+}
+
+// ---- family order ---------------------------------------------------------------
+// Slot 0 holds the root, and the children of node v are the slots 1 + k0[v] .. in Morton
+// order, k0 the exclusive prefix over pre-order of the nodes' child counts. Rank of node
+// v among its siblings (children of u):
+__device__ __forceinline__ int32_t sibling_rank(const Node *__restrict__ nodes, int32_t u,
+                                                int32_t v)
+{
+    if (nodes[u].t.shift == (uint32_t)kMaxDepth << 24) return v - u - 1; // a bucket's leaves
+    int32_t r = 0;
+    for (int32_t q = u + 1; q < v; q = nodes[q].t.escape) ++r; // at most seven before it
+    return r;
+}
+
+// Child counts: a node's last child (same escape) knows its own rank. Leaves have none.
+__global__ void family_count_kernel(const Node *__restrict__ nodes,
+                                    const int32_t *__restrict__ parent,
+                                    const int64_t *d_num_nodes, int32_t *__restrict__ count)
+{
+    const int64_t m = *d_num_nodes;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < m;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const NodeTopo t = nodes[v].t;
+        if (node_is_leaf(t.shift)) count[v] = 0;
+        const int32_t u = parent[v];
+        if (u >= 0 && nodes[u].t.escape == t.escape)
+            count[u] = sibling_rank(nodes, u, (int32_t)v) + 1;
+    }
+}
+
+__global__ void family_emit_kernel(const Node *__restrict__ nodes,
+                                   const int32_t *__restrict__ parent,
+                                   const int64_t *d_num_nodes, const int32_t *__restrict__ k0,
+                                   FamNode *__restrict__ fam)
+{
+    const int64_t m = *d_num_nodes;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < m;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const Node nd = nodes[v];
+        const int32_t u = parent[v];
+        const bool last = u < 0 || nodes[u].t.escape == nd.t.escape;
+        FamNode f;
+        f.cx = nd.g.cx;
+        f.cy = nd.g.cy;
+        f.cz = nd.g.cz;
+        f.cnt = nd.g.cnt;
+        f.pre = (int32_t)v;
+        f.up = u;
+        f.kids = node_is_leaf(nd.t.shift) ? 0u : (uint32_t)(1 + k0[v]);
+        f.shift = nd.t.shift | (last ? kLastSibling : 0u);
+        fam[u < 0 ? 0 : 1 + k0[u] + sibling_rank(nodes, u, (int32_t)v)] = f;
     }
 }
 
@@ -473,10 +986,10 @@ LenArgs make_args(relearn_ctx *c, const int32_t *vac_ax)
 {
     LenArgs a{};
     a.nodes = c->d_nodes;
+    a.fam = c->d_fam;
     a.pos = c->d_pos;
     a.perm = c->d_perm;
     a.act_src = c->d_act_src;
-    a.codes = c->d_codes;
     a.leaf_of = c->d_leaf;
     a.vac_ax = vac_ax;
     a.d_total = c->d_i64 + I64_ACTIVE;
@@ -493,11 +1006,8 @@ cudaError_t launch_length(relearn_ctx *c, const LenArgs &a, cudaStream_t st)
 {
     cudaError_t e;
     if ((e = cudaMemsetAsync(c->d_i32 + I32_WORK, 0, sizeof(int32_t), st))) return e;
-    void (*kern)(LenArgs) = length_kernel<kBack>;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0))) return e;
-    if (per_sm < 1) per_sm = 1;
-    kern<<<c->num_sms * per_sm, 256, 0, st>>>(a);
+    length_kernel<kBack>
+        <<<c->num_sms * RELEARN_LEN_MIN_BLOCKS, 32 * kGroupWarps, 0, st>>>(a);
     note_launch();
     return cudaGetLastError();
 }
@@ -518,6 +1028,20 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
         return e;
     len_fill_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(flag, c->d_act_off, n,
                                                                    c->d_act_src);
+    note_launch();
+    // the tree in family order, with the geometry the bottom-up update just formed (its
+    // prefix scratch is free again)
+    int32_t *k0 = reinterpret_cast<int32_t *>(c->d_acc);
+    const unsigned gm = grid_for(2 * n + 1, 256, c->num_sms);
+    family_count_kernel<<<gm, 256, 0, st>>>(c->d_nodes, c->d_parent, c->d_i64 + I64_NODES, k0);
+    note_launch();
+    // the node count as int32 (its low word)
+    if ((e = scan_exclusive(k0, k0, 2 * n + 1,
+                            reinterpret_cast<const int32_t *>(c->d_i64 + I64_NODES), nullptr,
+                            c->scan, st)))
+        return e;
+    family_emit_kernel<<<gm, 256, 0, st>>>(c->d_nodes, c->d_parent, c->d_i64 + I64_NODES, k0,
+                                           c->d_fam);
     note_launch();
     if ((e = cudaMemsetAsync(c->d_lsum, 0, 4 * sizeof(double), st))) return e;
     if ((e = launch_length<false>(c, make_args(c, vac_ax), st))) return e;
