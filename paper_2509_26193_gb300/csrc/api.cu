@@ -274,6 +274,8 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(scan.flags, scan_blocks + 3);
 #undef A
     if (e == cudaSuccess) {
+        for (auto init : {octree_init, search_init, synapses_init})
+            if (e == cudaSuccess) e = init();
         c->scan.max_blocks = scan_blocks;
         c->scan.status = c->d_status;
         c->scan.grid_cap = scan_grid_cap(c->num_sms);
@@ -436,9 +438,14 @@ relearn_status relearn_update_connectivity(relearn_ctx *c, const relearn_params 
     CK(search_run(c, *p, vac_ax, st), "search");
     if (ring) CK(record_phase(c->kev[c->nkev++][1], st), "event");
     if (timed) CK(record_phase(c->ev[3], st), "event");
-    CK(accept_requests(c, *p, vac_de, st), "accept");
-    if (timed) CK(record_phase(c->ev[4], st), "event");
-    CK(apply_requests(c, vac_ax, vac_de, type, st), "apply");
+    if (small_network(c)) { // one launch: its time counts as the acceptance's
+        CK(accept_apply_small(c, *p, vac_ax, vac_de, type, st), "accept and apply");
+        if (timed) CK(record_phase(c->ev[4], st), "event");
+    } else {
+        CK(accept_requests(c, *p, vac_de, st), "accept");
+        if (timed) CK(record_phase(c->ev[4], st), "event");
+        CK(apply_requests(c, vac_ax, vac_de, type, st), "apply");
+    }
     if (timed) CK(record_phase(c->ev[5], st), "event");
     c->diag_valid = (p->flags & RELEARN_FLAG_DIAG) != 0;
     c->stats_valid = true;

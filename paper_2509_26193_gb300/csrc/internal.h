@@ -150,6 +150,15 @@ enum { I32_N = 0, I32_Q, I32_NSYN, I32_NEW, I32_NODES, I32_WORK, I32_ACTIVE, I32
 
 namespace rl {
 
+// Whether a context's passes over its neurons and synapses run as one cluster kernel each
+// (cluster.cuh): by its sizes and capacities, since the counts of searches and synapses
+// are known on the device only.
+constexpr int64_t kSmallN = 40960, kSmallItems = 8 * kSmallN;
+inline bool small_network(const relearn_ctx *c)
+{
+    return c->n <= kSmallN && c->max_searches <= kSmallItems && c->max_synapses <= kSmallItems;
+}
+
 // Blocks for a grid-stride loop over n items: enough to cover n, at most 32 per SM.
 inline unsigned grid_for(int64_t n, int threads, int num_sms)
 {
@@ -184,6 +193,11 @@ cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int32_t *vals, in
                            cudaStream_t st, int *which);
 int64_t sort_blocks_needed(int64_t max_n);
 
+// Launch attributes of each file's cluster kernels on the current device.
+cudaError_t octree_init();
+cudaError_t search_init();
+cudaError_t synapses_init();
+
 // octree.cu -----------------------------------------------------------------
 cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, const float *y,
                          const float *z, const float *box_lo, const float *box_hi,
@@ -212,6 +226,9 @@ cudaError_t accept_requests(relearn_ctx *c, const relearn_params &p, const int32
                             cudaStream_t st);
 cudaError_t apply_requests(relearn_ctx *c, int32_t *vac_ax, int32_t *vac_de, const uint8_t *type,
                            cudaStream_t st);
+// Both in one launch, for small networks.
+cudaError_t accept_apply_small(relearn_ctx *c, const relearn_params &p, int32_t *vac_ax,
+                               int32_t *vac_de, const uint8_t *type, cudaStream_t st);
 // Typed dendrite pools: out[i] = vac_ax[i] where type[i] == kind, else 0; and back.
 cudaError_t select_type(relearn_ctx *c, const int32_t *vac_ax, const uint8_t *type, int kind,
                         int32_t *out, cudaStream_t st);

@@ -17,6 +17,7 @@
 // entries and rounds its centroid once to FP32 (see inner_sums).
 #include <mutex>
 
+#include "cluster.cuh"
 #include "internal.h"
 
 namespace rl {
@@ -661,9 +662,9 @@ __device__ __forceinline__ float centroid_coord(int64_t s, int64_t c, float cf, 
     return __fadd_rn(h3, lo);
 }
 
-__device__ __forceinline__ void inner_sums(Node *__restrict__ nodes, int64_t v, int64_t first,
-                                           int64_t size, const L4 *__restrict__ P,
-                                           const Geom *g)
+// (P without __restrict__: reduce_small_kernel writes it in the same launch)
+__device__ __forceinline__ void inner_sums(Node *nodes, int64_t v, int64_t first, int64_t size,
+                                           const L4 *P, const Geom *g)
 {
     const L4 s = l4_sub(P[first + size], P[first]);
     if (s.c > 0) {
@@ -706,6 +707,58 @@ __global__ void reduce_nodes_kernel(Node *__restrict__ nodes, const int32_t *__r
         if (size < 2) continue;
         const int32_t first = nodes[v].t.neuron;
         inner_sums(nodes, v, first, size, P, g_all + net_at(net, first));
+    }
+}
+
+// The whole bottom-up update of a small network (see cluster.cuh): leaves and prefix in
+// one scan, then the inner nodes. The sums are exact integers, so the result does not
+// depend on the form.
+__device__ __forceinline__ L4 add(L4 x, L4 y) { return l4_add(x, y); }
+__device__ __forceinline__ L4 up(L4 x, int o) { return l4_shfl_up(x, o); }
+
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads)
+    reduce_small_kernel(Node *nodes, const int32_t *leaf_of, const int32_t *perm,
+                        const float4 *pos, const int4 *posq, const int32_t *vac_de, int64_t n,
+                        L4 *P, const int32_t *nsize, const int64_t *d_num_nodes,
+                        const int32_t *net, const Geom *g_all, const int32_t *root,
+                        const int64_t *off, int32_t B)
+{
+    namespace cf = cluster_form;
+    auto weight = [&](int64_t s, int32_t c) {
+        const int4 q = posq[s];
+        const long long lc = c;
+        return L4{lc, lc * q.x, lc * q.y, lc * q.z};
+    };
+    const L4 total = cf::scan<L4>(
+        n,
+        [&](int64_t s) {
+            const int32_t c = max(vac_de[perm[s]], 0);
+            const float4 p = pos[s];
+            const int32_t v = leaf_of[s];
+            Node nd;
+            nd.g = c > 0 ? NodeGeo{p.x, p.y, p.z, (float)c} : NodeGeo{0.f, 0.f, 0.f, 0.f};
+            nd.t = NodeTopo{v + 1, kLeafShift, (int32_t)s, c};
+            nodes[v] = nd;
+            return weight(s, c);
+        },
+        [&](int64_t s) { return weight(s, max(vac_de[perm[s]], 0)); },
+        [&](int64_t s, L4 prefix, L4, L4) { P[s] = prefix; });
+    const int64_t tid = cf::first();
+    if (tid == 0) P[n] = total;
+    cf::sync();
+    const int64_t m = *d_num_nodes;
+    for (int64_t b = tid; b < B; b += cf::kStride) { // a root above one leaf
+        const int32_t v = B > 1 ? root[b] : 0;
+        const int64_t from = B > 1 ? off[b] : 0, last = B > 1 ? off[b + 1] : n;
+        if (last - from < 2 && !node_is_leaf(nodes[v].t.shift))
+            inner_sums(nodes, v, from, last - from, P, g_all + b);
+    }
+    for (int64_t v = tid; v < m; v += cf::kStride) {
+        const int32_t size = nsize[v];
+        if (size < 2) continue;
+        const int32_t from = nodes[v].t.neuron;
+        inner_sums(nodes, v, from, size, P, g_all + net_at(net, from));
     }
 }
 
@@ -788,12 +841,22 @@ cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, c
     return cudaGetLastError();
 }
 
+cudaError_t octree_init() { return cluster_form::allow(reduce_small_kernel); }
+
 cudaError_t octree_reduce(relearn_ctx *c, const int32_t *vac_de, cudaStream_t st)
 {
     const int64_t n = c->n;
     const int64_t nb = (n + kRedTile - 1) / kRedTile;
     L4 *P = reinterpret_cast<L4 *>(c->d_acc); // n + 1 prefix entries
     L4 *tile = P + (n + 1);                     // nb tile sums, then tile prefixes
+    if (small_network(c)) {
+        reduce_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+            c->d_nodes, c->d_leaf, c->d_perm, c->d_pos, c->d_posq, vac_de, n, P, c->d_nsize,
+            c->d_i64 + I64_NODES, c->num_nets > 1 ? c->d_net : nullptr, c->d_geom, c->d_root,
+            c->d_off, c->num_nets);
+        note_launch();
+        return cudaGetLastError();
+    }
     if (nb > 0) {
         reduce_leaves_kernel<<<(unsigned)nb, 256, 0, st>>>(c->d_nodes, c->d_leaf, c->d_perm,
                                                             c->d_pos, c->d_posq, vac_de, n, tile);

@@ -38,6 +38,7 @@
 // exponents shifted by the nearest candidate's d^2 (an exact common factor).
 #include <cooperative_groups.h>
 
+#include "cluster.cuh"
 #include "internal.h"
 #include "scan_pair.cuh"
 
@@ -175,6 +176,32 @@ struct QueryOp {
         *d_Qsum += void_ ? 0 : q;
     }
 };
+
+// The query setup of a small network (see cluster.cuh); work and failed are the search's
+// counters, set to zero here.
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads) query_small_kernel(QueryOp op, int32_t *work,
+                                                                 int64_t *failed)
+{
+    namespace cf = cluster_form;
+    const int64_t tid = cf::first();
+    op.prologue(tid, cf::kStride);
+    auto load = [&](int64_t k) {
+        const int2 v = op.load(k);
+        return cf::I64x2{v.x, v.y};
+    };
+    const cf::I64x2 total = cf::scan<cf::I64x2>(
+        op.n, load, load, [&](int64_t k, cf::I64x2 prefix, cf::I64x2 v, cf::I64x2) {
+            op.emit(k, prefix.a, prefix.b, make_int2((int)v.a, (int)v.b));
+        });
+    if (tid == 0) { // every prologue ran before the scan's barrier
+        *work = 0;
+        *failed = 0;
+        op.store_totals(total.a, total.b);
+        op.finish();
+    }
+    cf::sync();
+}
 
 struct SearchArgs {
     const Node *__restrict__ nodes;
@@ -1119,6 +1146,8 @@ cudaError_t search_constants(relearn_ctx *c, const relearn_params &p, cudaStream
     return cudaGetLastError();
 }
 
+cudaError_t search_init() { return cluster_form::allow(query_small_kernel); }
+
 cudaError_t search_prepare(relearn_ctx *c, const relearn_params &p, const int32_t *vac_ax,
                            cudaStream_t st)
 {
@@ -1147,6 +1176,16 @@ cudaError_t search_prepare(relearn_ctx *c, const relearn_params &p, const int32_
     op.net_sigma = p.net_sigma;
     op.net_theta = p.net_theta;
     op.sc_all = c->d_sc;
+    // (the stalled-scan hook needs the single-pass scan)
+    if (small_network(c) && c->debug_stall_tile < 0) {
+        query_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+            op, c->d_i32 + I32_WORK, c->d_i64 + I64_FAILED);
+        note_launch();
+        return cudaGetLastError();
+    }
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(c->d_i32 + I32_WORK, 0, sizeof(int32_t), st))) return e;
+    if ((e = cudaMemsetAsync(c->d_i64 + I64_FAILED, 0, sizeof(int64_t), st))) return e;
     const int64_t tiles = std::max<int64_t>(1, (n + pair_scan::kTile - 1) / pair_scan::kTile);
     if (tiles > c->scan.max_blocks) return cudaErrorInvalidValue;
     pair_scan::scan_pair_kernel<QueryOp><<<(unsigned)tiles, pair_scan::kThreads, 0, st>>>(
@@ -1172,8 +1211,6 @@ cudaError_t search_run(relearn_ctx *c, const relearn_params &p, const int32_t *v
                        cudaStream_t st)
 {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(c->d_i32 + I32_WORK, 0, sizeof(int32_t), st))) return e;
-    if ((e = cudaMemsetAsync(c->d_i64 + I64_FAILED, 0, sizeof(int64_t), st))) return e;
     SearchArgs a;
     a.nodes = c->d_nodes;
     a.pos = c->d_pos;
@@ -1251,11 +1288,18 @@ cudaError_t search_run(relearn_ctx *c, const relearn_params &p, const int32_t *v
     const int64_t warps = (int64_t)c->num_sms * per_sm * 8;
     auto cap = [](int64_t v) { return (int32_t)std::min<int64_t>(v, 1 << 30); };
     a.split_below = sg >= 3000 ? cap((int64_t)(sg - 3000) * 1024) : cap(warps * kSplitWaves);
-    // exactly one of the two kernels does the work (each reads the source count)
-    kern<<<c->num_sms * per_sm, 256, 0, st>>>(a);
-    note_launch();
-    split<<<c->num_sms * per_sm_split, 256, split_smem, st>>>(a);
-    note_launch();
+    // exactly one of the two kernels does the work (each reads the source count); one that
+    // cannot be it, whatever the count, is not launched
+    const bool may_union = a.forced_group != 2 && (a.forced_group != 0 || c->n > a.split_below);
+    const bool may_split = a.forced_group == 2 || a.forced_group == 0;
+    if (may_union) {
+        kern<<<c->num_sms * per_sm, 256, 0, st>>>(a);
+        note_launch();
+    }
+    if (may_split) {
+        split<<<c->num_sms * per_sm_split, 256, split_smem, st>>>(a);
+        note_launch();
+    }
     if (a.defer) {
         // regroup the deferred restarts by drawn node, then finish them
         int bits = 1;

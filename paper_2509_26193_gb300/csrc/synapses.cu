@@ -16,6 +16,7 @@
 // or an export needs it. Spike delivery reads the store in any order: each
 // synapse of a spiking source adds its sign to its target with an integer atomic
 // (exact, so the order does not matter).
+#include "cluster.cuh"
 #include "internal.h"
 
 namespace rl {
@@ -72,8 +73,23 @@ __global__ void accept_scatter_kernel(const int32_t *d_Q, const int32_t *__restr
     }
 }
 
-// A target's request count is the difference of neighbouring bucket offsets (one
-// read of two adjacent words).
+// Whether request r to target t is accepted. A target's request count is the difference
+// of neighbouring bucket offsets (one read of two adjacent words).
+__device__ __forceinline__ bool accepted(int64_t r, int32_t t, const uint32_t *prio,
+                                         const int32_t *toff, const uint64_t *bucket,
+                                         const int32_t *vac_de)
+{
+    const int32_t v = max(vac_de[t], 0);
+    const int32_t o = toff[t], rt = toff[t + 1] - o;
+    if (rt <= v) return true;
+    if (v == 0) return false;
+    const uint64_t kr = request_key(prio[r], r); // keys are distinct
+    const uint64_t *bk = bucket + o;
+    int32_t below = 0;
+    for (int32_t k = 0; k < rt && below < v; ++k) below += bk[k] < kr ? 1 : 0;
+    return below < v;
+}
+
 __global__ void accept_decide_kernel(const int32_t *d_Q, const int32_t *__restrict__ req_tgt,
                                      const uint32_t *__restrict__ prio,
                                      const int32_t *__restrict__ toff,
@@ -86,21 +102,10 @@ __global__ void accept_decide_kernel(const int32_t *d_Q, const int32_t *__restri
     int64_t dec = 0;
     GRID_STRIDE(r, Q)
     {
-        int32_t t = req_tgt[r];
+        const int32_t t = req_tgt[r];
         uint8_t a = 0;
         if (t >= 0) {
-            int32_t v = vac_de[t];
-            if (v < 0) v = 0;
-            const int32_t o = toff[t], rt = toff[t + 1] - o;
-            if (rt <= v) {
-                a = 1;
-            } else if (v > 0) {
-                const uint64_t kr = request_key(prio[r], r); // keys are distinct
-                const uint64_t *bk = bucket + o;
-                int32_t below = 0;
-                for (int32_t k = 0; k < rt && below < v; ++k) below += bk[k] < kr ? 1 : 0;
-                a = below < v ? 1 : 0;
-            }
+            a = accepted(r, t, prio, toff, bucket, vac_de) ? 1 : 0;
             dec += a ? 0 : 1;
         }
         acc[r] = a;
@@ -194,7 +199,7 @@ __global__ void degree_kernel(const int32_t *d_nsyn, const int32_t *__restrict__
 // identical (the sign follows the source), so their order does not matter.
 __global__ void row_scatter_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
                                    const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
-                                   const int32_t *__restrict__ out_ptr, int32_t *__restrict__ fill,
+                                   const int32_t *__restrict__ out_ptr, int32_t *__restrict__ left,
                                    int32_t *__restrict__ row_src, int32_t *__restrict__ row_tgt,
                                    int32_t *__restrict__ row_sign)
 {
@@ -202,11 +207,25 @@ __global__ void row_scatter_kernel(const int32_t *d_nsyn, const int32_t *__restr
     GRID_STRIDE(k, m)
     {
         const int32_t s = src[k];
-        const int32_t r = out_ptr[s] + atomicAdd(&fill[s], 1);
+        const int32_t r = out_ptr[s] + atomicSub(&left[s], 1) - 1;
         row_src[r] = s;
         row_tgt[r] = tgt[k];
         row_sign[r] = sign[k];
     }
+}
+
+// Where record r of a row belongs: its rank in the row by (target, place in the row).
+__device__ __forceinline__ int32_t row_place(int64_t r, const int32_t *row_src,
+                                             const int32_t *row_tgt, const int32_t *out_ptr)
+{
+    const int32_t s = row_src[r], t = row_tgt[r];
+    const int32_t b = out_ptr[s], e = out_ptr[s + 1];
+    int32_t rank = 0;
+    for (int32_t j = b; j < e; ++j) {
+        const int32_t tj = row_tgt[j];
+        rank += (tj < t || (tj == t && j < r)) ? 1 : 0;
+    }
+    return b + rank;
 }
 
 __global__ void row_rank_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ row_src,
@@ -218,16 +237,9 @@ __global__ void row_rank_kernel(const int32_t *d_nsyn, const int32_t *__restrict
     const int64_t m = *d_nsyn;
     GRID_STRIDE(r, m)
     {
-        const int32_t s = row_src[r], t = row_tgt[r];
-        const int32_t b = out_ptr[s], e = out_ptr[s + 1];
-        int32_t rank = 0;
-        for (int32_t j = b; j < e; ++j) {
-            const int32_t tj = row_tgt[j];
-            rank += (tj < t || (tj == t && j < r)) ? 1 : 0;
-        }
-        const int32_t w = b + rank;
-        src[w] = s;
-        tgt[w] = t;
+        const int32_t w = row_place(r, row_src, row_tgt, out_ptr);
+        src[w] = row_src[r];
+        tgt[w] = row_tgt[r];
         sign[w] = (int8_t)row_sign[r];
     }
 }
@@ -235,15 +247,25 @@ __global__ void row_rank_kernel(const int32_t *d_nsyn, const int32_t *__restrict
 // In-view: synapse numbers k (canonical order) grouped by target, each row ordered by
 // k (i.e. by source), by the same scatter-then-rank.
 __global__ void in_scatter_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ tgt,
-                                  const int32_t *__restrict__ in_ptr, int32_t *__restrict__ fill,
+                                  const int32_t *__restrict__ in_ptr, int32_t *__restrict__ left,
                                   int32_t *__restrict__ row_k)
 {
     const int64_t m = *d_nsyn;
     GRID_STRIDE(k, m)
     {
         const int32_t t = tgt[k];
-        row_k[in_ptr[t] + atomicAdd(&fill[t], 1)] = (int32_t)k;
+        row_k[in_ptr[t] + atomicSub(&left[t], 1) - 1] = (int32_t)k;
     }
+}
+
+__device__ __forceinline__ int32_t in_place(int64_t r, const int32_t *row_k, const int32_t *tgt,
+                                            const int32_t *in_ptr)
+{
+    const int32_t k = row_k[r], t = tgt[k];
+    const int32_t b = in_ptr[t], e = in_ptr[t + 1];
+    int32_t rank = 0;
+    for (int32_t j = b; j < e; ++j) rank += row_k[j] < k ? 1 : 0;
+    return b + rank;
 }
 
 __global__ void in_rank_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ tgt,
@@ -253,15 +275,21 @@ __global__ void in_rank_kernel(const int32_t *d_nsyn, const int32_t *__restrict_
     const int64_t m = *d_nsyn;
     GRID_STRIDE(r, m)
     {
-        const int32_t k = row_k[r], t = tgt[k];
-        const int32_t b = in_ptr[t], e = in_ptr[t + 1];
-        int32_t rank = 0;
-        for (int32_t j = b; j < e; ++j) rank += row_k[j] < k ? 1 : 0;
-        in_syn[b + rank] = k;
+        in_syn[in_place(r, row_k, tgt, in_ptr)] = row_k[r];
     }
 }
 
 // ---------------------------------------------------------------- deletion
+// Neuron i retracts vacant elements first; what is left breaks bound ones.
+__device__ __forceinline__ int32_t retract(int64_t i, const int32_t *retract_, int32_t *vac,
+                                           int32_t degree)
+{
+    const int32_t r = max(retract_[i], 0), v = vac[i];
+    const int32_t t = r < v ? r : max(v, 0);
+    vac[i] = v - t;
+    return min(r - t, degree);
+}
+
 __global__ void delete_needs_kernel(int64_t n, const int32_t *__restrict__ retract_ax,
                                     const int32_t *__restrict__ retract_de, int32_t *vac_ax,
                                     int32_t *vac_de, const int32_t *__restrict__ out_ptr,
@@ -270,21 +298,25 @@ __global__ void delete_needs_kernel(int64_t n, const int32_t *__restrict__ retra
 {
     GRID_STRIDE(i, n)
     {
-        int32_t ra = retract_ax[i] > 0 ? retract_ax[i] : 0;
-        int32_t va = vac_ax[i];
-        int32_t ta = ra < va ? ra : (va > 0 ? va : 0);
-        vac_ax[i] = va - ta;
-        ra -= ta;
-        int32_t deg = out_ptr[i + 1] - out_ptr[i];
-        need_ax[i] = ra < deg ? ra : deg;
-        int32_t rd = retract_de[i] > 0 ? retract_de[i] : 0;
-        int32_t vd = vac_de[i];
-        int32_t td = rd < vd ? rd : (vd > 0 ? vd : 0);
-        vac_de[i] = vd - td;
-        rd -= td;
-        int32_t din = in_ptr[i + 1] - in_ptr[i];
-        need_de[i] = rd < din ? rd : din;
+        need_ax[i] = retract(i, retract_ax, vac_ax, out_ptr[i + 1] - out_ptr[i]);
+        need_de[i] = retract(i, retract_de, vac_de, in_ptr[i + 1] - in_ptr[i]);
     }
+}
+
+// The priority of slot k of its out-row and of its in-row, where the row breaks some of
+// its slots but not all (select_row reads no others).
+__device__ __forceinline__ void slot_priorities(int64_t k, const int32_t *src, const int32_t *tgt,
+                                                const int32_t *in_syn, const int32_t *out_ptr,
+                                                const int32_t *in_ptr, const int32_t *need_ax,
+                                                const int32_t *need_de, uint32_t *prio_ax,
+                                                uint32_t *prio_de, uint64_t seed, uint32_t step)
+{
+    const int32_t i = src[k], wi = need_ax[i], bi = out_ptr[i];
+    if (wi > 0 && wi < out_ptr[i + 1] - bi)
+        prio_ax[k] = philox_x((uint32_t)i, step, (uint32_t)(k - bi), 2u, seed);
+    const int32_t j = tgt[in_syn[k]], wj = need_de[j], bj = in_ptr[j];
+    if (wj > 0 && wj < in_ptr[j + 1] - bj)
+        prio_de[k] = philox_x((uint32_t)j, step, (uint32_t)(k - bj), 3u, seed);
 }
 
 __global__ void delete_prio_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
@@ -292,6 +324,8 @@ __global__ void delete_prio_kernel(const int32_t *d_nsyn, const int32_t *__restr
                                    const int32_t *__restrict__ tgt,
                                    const int32_t *__restrict__ out_ptr,
                                    const int32_t *__restrict__ in_ptr,
+                                   const int32_t *__restrict__ need_ax,
+                                   const int32_t *__restrict__ need_de,
                                    uint32_t *__restrict__ prio_ax, uint32_t *__restrict__ prio_de,
                                    uint8_t *__restrict__ sel_ax, uint8_t *__restrict__ sel_de,
                                    uint64_t seed, uint32_t step)
@@ -299,16 +333,33 @@ __global__ void delete_prio_kernel(const int32_t *d_nsyn, const int32_t *__restr
     const int64_t m = *d_nsyn;
     GRID_STRIDE(k, m)
     {
-        int32_t i = src[k];
-        prio_ax[k] = philox_x((uint32_t)i, step, (uint32_t)(k - out_ptr[i]), 2u, seed);
-        int32_t j = tgt[in_syn[k]];
-        prio_de[k] = philox_x((uint32_t)j, step, (uint32_t)(k - in_ptr[j]), 3u, seed);
+        slot_priorities(k, src, tgt, in_syn, out_ptr, in_ptr, need_ax, need_de, prio_ax, prio_de,
+                        seed, step);
         sel_ax[k] = 0;
         sel_de[k] = 0;
     }
 }
 
-// Row i picks its `need` slots with the smallest (priority, slot).
+// Row i picks its `want` slots with the smallest (priority, slot).
+__device__ __forceinline__ void select_row(int32_t b, int32_t deg, int32_t want,
+                                           const uint32_t *prio, const int32_t *map, uint8_t *sel)
+{
+    if (want <= 0) return;
+    for (int32_t k = 0; k < deg; ++k) {
+        bool take = want >= deg; // all of them
+        if (!take) {
+            const uint32_t pk = prio[b + k];
+            int32_t below = 0;
+            for (int32_t o = 0; o < deg && below < want; ++o) {
+                const uint32_t po = prio[b + o];
+                if (po < pk || (po == pk && o < k)) ++below;
+            }
+            take = below < want;
+        }
+        if (take) sel[map ? map[b + k] : b + k] = 1;
+    }
+}
+
 __global__ void delete_select_kernel(int64_t n, const int32_t *__restrict__ ptr,
                                      const int32_t *__restrict__ need,
                                      const uint32_t *__restrict__ prio,
@@ -316,18 +367,8 @@ __global__ void delete_select_kernel(int64_t n, const int32_t *__restrict__ ptr,
 {
     GRID_STRIDE(i, n)
     {
-        const int32_t want = need[i];
-        if (want <= 0) continue;
-        const int32_t b = ptr[i], deg = ptr[i + 1] - b;
-        for (int32_t k = 0; k < deg; ++k) {
-            const uint32_t pk = prio[b + k];
-            int32_t below = 0;
-            for (int32_t o = 0; o < deg && below < want; ++o) {
-                uint32_t po = prio[b + o];
-                if (po < pk || (po == pk && o < k)) ++below;
-            }
-            if (below < want) sel[map ? map[b + k] : b + k] = 1;
-        }
+        const int32_t b = ptr[i];
+        select_row(b, ptr[i + 1] - b, need[i], prio, map, sel);
     }
 }
 
@@ -390,6 +431,13 @@ __global__ void spikes_kernel(const int32_t *d_nsyn, const int32_t *__restrict__
 // source s whether s spiked, spiked iff philox({s, t, step, 4}).x < rate[s] * 2^32
 // (an exact FP64 comparison); duplicates of (s, t) share that decision (each
 // copy computes the same word).
+__device__ __forceinline__ bool rate_fires(int32_t s, int32_t t, float rate, uint64_t seed,
+                                           uint32_t step)
+{
+    const uint32_t w = philox_x((uint32_t)s, (uint32_t)t, step, 4u, seed);
+    return (double)w < (double)rate * 4294967296.0;
+}
+
 __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
                              const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
                              const float *__restrict__ rate, uint64_t seed, uint32_t step,
@@ -399,8 +447,243 @@ __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ 
     GRID_STRIDE(k, m)
     {
         const int32_t s = src[k], t = tgt[k];
-        const uint32_t w = philox_x((uint32_t)s, (uint32_t)t, step, 4u, seed);
-        if ((double)w < (double)rate[s] * 4294967296.0) atomicAdd(&input[t], (int32_t)sign[k]);
+        if (rate_fires(s, t, rate[s], seed, step)) atomicAdd(&input[t], (int32_t)sign[k]);
+    }
+}
+
+// ---------------------------------------------------------------- small networks
+// The steps above for a small network, one launch per call (see cluster.cuh): the same
+// arithmetic and, where an order matters, the same order. Pointers without __restrict__:
+// one step reads what another wrote in the same launch.
+#define CLUSTER_STRIDE(i, n)                                                                      \
+    for (int64_t i = cluster_form::first(); i < (n); i += cluster_form::kStride)
+
+struct StoreArgs {
+    int64_t n, max_synapses;
+    int32_t *d_nsyn;
+    int64_t *d_nsyn64;
+    int32_t *src, *tgt;
+    int8_t *sign;
+    uint64_t seed;
+    uint32_t step;
+};
+
+StoreArgs store_args(relearn_ctx *c, uint64_t seed, uint32_t step)
+{
+    return StoreArgs{c->n,         c->max_synapses, c->d_i32 + I32_NSYN, c->d_i64 + I64_NSYN,
+                     c->d_syn_src, c->d_syn_tgt,    c->d_syn_sign,       seed,
+                     step};
+}
+
+struct AcceptArgs {
+    const int32_t *d_Q;
+    int32_t *status;
+    const int32_t *req_src, *req_elem, *req_tgt;
+    uint32_t *prio;
+    int32_t *tcnt, *toff;
+    uint64_t *bucket;
+    uint8_t *acc;
+    int64_t *declined, *formed;
+    int32_t *vac_ax, *vac_de;
+    const uint8_t *type;
+};
+
+// Acceptance and apply of an update.
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads) accept_apply_small_kernel(AcceptArgs a, StoreArgs st)
+{
+    namespace cf = cluster_form;
+    const int64_t Q = *a.d_Q;
+    const int64_t base = *st.d_nsyn;
+    const bool failed = *(volatile int32_t *)a.status != 0; // an earlier kernel's error
+    CLUSTER_STRIDE(i, st.n + 1) a.tcnt[i] = 0;
+    if (cf::first() == 0) *a.declined = 0;
+    cf::sync();
+    CLUSTER_STRIDE(r, Q)
+    {
+        const int32_t t = a.req_tgt[r];
+        if (t < 0) continue;
+        atomicAdd(&a.tcnt[t], 1);
+        a.prio[r] = philox_x((uint32_t)a.req_src[r], st.step,
+                             ((uint32_t)a.req_elem[r] << 8) | 0xFFu, 1u, st.seed);
+    }
+    cf::sync();
+    auto count = [&](int64_t i) { return cf::I32{a.tcnt[i]}; };
+    cf::scan<cf::I32>(st.n + 1, count, count, [&](int64_t i, cf::I32 prefix, cf::I32, cf::I32) {
+        a.toff[i] = prefix.v;
+    });
+    cf::sync();
+    CLUSTER_STRIDE(r, Q)
+    {
+        const int32_t t = a.req_tgt[r];
+        if (t >= 0)
+            a.bucket[a.toff[t] + atomicSub(&a.tcnt[t], 1) - 1] = request_key(a.prio[r], r);
+    }
+    cf::sync();
+    int64_t dec = 0;
+    // every decision is made before the first vacancy changes (the scan's barrier)
+    const cf::I32 formed = cf::scan<cf::I32>(
+        Q,
+        [&](int64_t r) {
+            const int32_t t = a.req_tgt[r];
+            const bool ok = t >= 0 && accepted(r, t, a.prio, a.toff, a.bucket, a.vac_de);
+            dec += t >= 0 && !ok ? 1 : 0;
+            a.acc[r] = ok ? 1 : 0;
+            return cf::I32{ok ? 1 : 0};
+        },
+        [&](int64_t r) { return cf::I32{a.acc[r]}; },
+        [&](int64_t r, cf::I32 prefix, cf::I32 ok, cf::I32 total) {
+            // nothing is applied on overflow
+            if (!ok.v || failed || base + total.v > st.max_synapses) return;
+            const int32_t s = a.req_src[r], t = a.req_tgt[r];
+            atomicSub(&a.vac_ax[s], 1);
+            atomicSub(&a.vac_de[t], 1);
+            const int64_t k = base + prefix.v;
+            st.src[k] = s;
+            st.tgt[k] = t;
+            st.sign[k] = a.type[s] ? (int8_t)-1 : (int8_t)1;
+        });
+    for (int off = 16; off; off >>= 1) dec += __shfl_xor_sync(0xffffffffu, dec, off);
+    if ((threadIdx.x & 31) == 0 && dec)
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.declined), (unsigned long long)dec);
+    if (cf::first() == 0) {
+        const bool fits = base + formed.v <= st.max_synapses;
+        if (!failed && !fits) set_status(a.status, RELEARN_ERR_CAPACITY);
+        const int64_t f = failed || !fits ? 0 : formed.v;
+        *a.formed = f;
+        *st.d_nsyn = (int32_t)(base + f);
+        *st.d_nsyn64 = base + f;
+    }
+    cf::sync();
+}
+
+struct DeleteArgs {
+    bool canonical; // the views below are those of the store
+    int32_t *out_cnt, *in_cnt, *out_ptr, *in_ptr;
+    int32_t *row_src, *row_tgt, *row_sign, *row_k, *in_syn;
+    const int32_t *retract_ax, *retract_de;
+    int32_t *vac_ax, *vac_de, *need_ax, *need_de;
+    uint32_t *prio_ax, *prio_de;
+    uint8_t *sel_ax, *sel_de;
+    int64_t *broken;
+};
+
+// The canonical order and its views, then the deletion pass (see canonicalise_store and
+// delete_synapses).
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads) delete_small_kernel(DeleteArgs a, StoreArgs st)
+{
+    namespace cf = cluster_form;
+    const int64_t n = st.n, m = *st.d_nsyn;
+    if (!a.canonical) {
+        CLUSTER_STRIDE(i, n + 1) a.out_cnt[i] = a.in_cnt[i] = 0;
+        cf::sync();
+        CLUSTER_STRIDE(k, m)
+        {
+            atomicAdd(&a.out_cnt[st.src[k]], 1);
+            atomicAdd(&a.in_cnt[st.tgt[k]], 1);
+        }
+        cf::sync();
+        auto counts = [&](int64_t i) { return cf::I64x2{a.out_cnt[i], a.in_cnt[i]}; };
+        cf::scan<cf::I64x2>(n + 1, counts, counts,
+                            [&](int64_t i, cf::I64x2 prefix, cf::I64x2, cf::I64x2) {
+                                a.out_ptr[i] = (int32_t)prefix.a;
+                                a.in_ptr[i] = (int32_t)prefix.b;
+                            });
+        cf::sync();
+        CLUSTER_STRIDE(k, m)
+        {
+            const int32_t s = st.src[k];
+            const int32_t r = a.out_ptr[s] + atomicSub(&a.out_cnt[s], 1) - 1;
+            a.row_src[r] = s;
+            a.row_tgt[r] = st.tgt[k];
+            a.row_sign[r] = st.sign[k];
+        }
+        cf::sync();
+        CLUSTER_STRIDE(r, m)
+        {
+            const int32_t w = row_place(r, a.row_src, a.row_tgt, a.out_ptr);
+            st.src[w] = a.row_src[r];
+            st.tgt[w] = a.row_tgt[r];
+            st.sign[w] = (int8_t)a.row_sign[r];
+        }
+        cf::sync();
+        CLUSTER_STRIDE(k, m)
+        {
+            const int32_t t = st.tgt[k];
+            a.row_k[a.in_ptr[t] + atomicSub(&a.in_cnt[t], 1) - 1] = (int32_t)k;
+        }
+        cf::sync();
+        CLUSTER_STRIDE(r, m) a.in_syn[in_place(r, a.row_k, st.tgt, a.in_ptr)] = a.row_k[r];
+        cf::sync();
+    }
+    CLUSTER_STRIDE(i, n)
+    {
+        a.need_ax[i] = retract(i, a.retract_ax, a.vac_ax, a.out_ptr[i + 1] - a.out_ptr[i]);
+        a.need_de[i] = retract(i, a.retract_de, a.vac_de, a.in_ptr[i + 1] - a.in_ptr[i]);
+    }
+    cf::sync();
+    CLUSTER_STRIDE(k, m)
+    {
+        a.sel_ax[k] = 0;
+        a.sel_de[k] = 0;
+        slot_priorities(k, st.src, st.tgt, a.in_syn, a.out_ptr, a.in_ptr, a.need_ax, a.need_de,
+                        a.prio_ax, a.prio_de, st.seed, st.step);
+    }
+    cf::sync();
+    CLUSTER_STRIDE(i, n)
+    {
+        const int32_t b = a.out_ptr[i], d = a.in_ptr[i];
+        select_row(b, a.out_ptr[i + 1] - b, a.need_ax[i], a.prio_ax, nullptr, a.sel_ax);
+        select_row(d, a.in_ptr[i + 1] - d, a.need_de[i], a.prio_de, a.in_syn, a.sel_de);
+    }
+    cf::sync();
+    const cf::I32 kept = cf::scan<cf::I32>(
+        m,
+        [&](int64_t k) {
+            const bool x = a.sel_ax[k], d = a.sel_de[k];
+            if (x && !d) atomicAdd(&a.vac_de[st.tgt[k]], 1);
+            if (d && !x) atomicAdd(&a.vac_ax[st.src[k]], 1);
+            return cf::I32{x || d ? 0 : 1};
+        },
+        [&](int64_t k) { return cf::I32{a.sel_ax[k] || a.sel_de[k] ? 0 : 1}; },
+        [&](int64_t k, cf::I32 prefix, cf::I32 keep, cf::I32) {
+            if (!keep.v) return;
+            a.row_src[prefix.v] = st.src[k];
+            a.row_tgt[prefix.v] = st.tgt[k];
+            a.row_sign[prefix.v] = st.sign[k];
+        });
+    cf::sync();
+    CLUSTER_STRIDE(w, kept.v)
+    {
+        st.src[w] = a.row_src[w];
+        st.tgt[w] = a.row_tgt[w];
+        st.sign[w] = (int8_t)a.row_sign[w];
+    }
+    if (cf::first() == 0) {
+        *a.broken = m - kept.v;
+        *st.d_nsyn = kept.v;
+        *st.d_nsyn64 = kept.v;
+    }
+}
+
+// input = 0, then as spikes_kernel (spiked given) or rates_kernel.
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads)
+    deliver_small_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
+                         const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
+                         const uint8_t *__restrict__ spiked, const float *__restrict__ rate,
+                         uint64_t seed, uint32_t step, int64_t n, int32_t *input)
+{
+    namespace cf = cluster_form;
+    const int64_t m = *d_nsyn;
+    CLUSTER_STRIDE(i, n) input[i] = 0;
+    cf::sync();
+    CLUSTER_STRIDE(k, m)
+    {
+        const int32_t s = src[k];
+        const bool fires = spiked ? spiked[s] != 0 : rate_fires(s, tgt[k], rate[s], seed, step);
+        if (fires) atomicAdd(&input[tgt[k]], (int32_t)sign[k]);
     }
 }
 
@@ -409,6 +692,13 @@ __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ 
 cudaError_t deliver_rates(relearn_ctx *c, const float *rate, uint64_t seed, uint32_t step,
                           int32_t *input, cudaStream_t st)
 {
+    if (small_network(c)) {
+        deliver_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+            c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, nullptr, rate, seed, step, c->n,
+            input);
+        note_launch();
+        return cudaGetLastError();
+    }
     cudaError_t e;
     if ((e = cudaMemsetAsync(input, 0, c->n * sizeof(int32_t), st))) return e;
     rates_kernel<<<grid_for(c->max_synapses, 256, c->num_sms), 256, 0, st>>>(
@@ -450,7 +740,7 @@ cudaError_t canonicalise_store(relearn_ctx *c, cudaStream_t st)
     const int64_t n = c->n;
     const int32_t *dm = c->d_i32 + I32_NSYN;
     const unsigned gs = grid_for(c->max_synapses, 256, c->num_sms);
-    int32_t *out_cnt = c->d_cnt, *in_cnt = c->d_tcnt, *fill = c->d_need_ax;
+    int32_t *out_cnt = c->d_cnt, *in_cnt = c->d_tcnt;
     int32_t *row_src = c->d_val, *row_sign = c->d_val_alt;
     int32_t *row_tgt = reinterpret_cast<int32_t *>(c->d_key32);
     int32_t *row_k = reinterpret_cast<int32_t *>(c->d_key32_alt);
@@ -461,19 +751,51 @@ cudaError_t canonicalise_store(relearn_ctx *c, cudaStream_t st)
     if ((e = scan_exclusive(out_cnt, c->d_out_ptr, n + 1, nullptr, nullptr, c->scan, st)))
         return e;
     if ((e = scan_exclusive(in_cnt, c->d_in_ptr, n + 1, nullptr, nullptr, c->scan, st))) return e;
-    if ((e = cudaMemsetAsync(fill, 0, n * sizeof(int32_t), st))) return e;
     row_scatter_kernel<<<gs, 256, 0, st>>>(dm, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign,
-                                           c->d_out_ptr, fill, row_src, row_tgt, row_sign);
+                                           c->d_out_ptr, out_cnt, row_src, row_tgt, row_sign);
     note_launch();
     row_rank_kernel<<<gs, 256, 0, st>>>(dm, row_src, row_tgt, row_sign, c->d_out_ptr,
                                         c->d_syn_src, c->d_syn_tgt, c->d_syn_sign);
     note_launch();
-    if ((e = cudaMemsetAsync(fill, 0, n * sizeof(int32_t), st))) return e;
-    in_scatter_kernel<<<gs, 256, 0, st>>>(dm, c->d_syn_tgt, c->d_in_ptr, fill, row_k);
+    in_scatter_kernel<<<gs, 256, 0, st>>>(dm, c->d_syn_tgt, c->d_in_ptr, in_cnt, row_k);
     note_launch();
     in_rank_kernel<<<gs, 256, 0, st>>>(dm, c->d_syn_tgt, c->d_in_ptr, row_k, c->d_in_syn);
     note_launch();
     c->canonical = true;
+    return cudaGetLastError();
+}
+
+cudaError_t synapses_init()
+{
+    cudaError_t e;
+    if ((e = cluster_form::allow(accept_apply_small_kernel))) return e;
+    if ((e = cluster_form::allow(delete_small_kernel))) return e;
+    return cluster_form::allow(deliver_small_kernel);
+}
+
+cudaError_t accept_apply_small(relearn_ctx *c, const relearn_params &p, int32_t *vac_ax,
+                               int32_t *vac_de, const uint8_t *type, cudaStream_t st)
+{
+    AcceptArgs a;
+    a.d_Q = c->d_i32 + I32_Q;
+    a.status = c->d_status;
+    a.req_src = c->d_req_src;
+    a.req_elem = c->d_req_elem;
+    a.req_tgt = c->d_req_tgt;
+    a.prio = c->d_req_prio;
+    a.tcnt = c->d_tcnt;
+    a.toff = c->d_toff;
+    a.bucket = c->d_bucket;
+    a.acc = c->d_req_acc;
+    a.declined = c->d_i64 + I64_DECLINED;
+    a.formed = c->d_i64 + I64_FORMED;
+    a.vac_ax = vac_ax;
+    a.vac_de = vac_de;
+    a.type = type;
+    accept_apply_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+        a, store_args(c, p.seed, (uint32_t)p.step));
+    note_launch();
+    c->canonical = false; // as in apply_requests
     return cudaGetLastError();
 }
 
@@ -512,13 +834,43 @@ cudaError_t delete_synapses(relearn_ctx *c, const relearn_params &p, const int32
     const int32_t *dm = c->d_i32 + I32_NSYN;
     const unsigned gs = grid_for(c->max_synapses, 256, c->num_sms);
     const unsigned gn = grid_for(n, 256, c->num_sms);
+    if (small_network(c)) {
+        DeleteArgs a;
+        a.canonical = c->canonical;
+        a.out_cnt = c->d_cnt;
+        a.in_cnt = c->d_tcnt;
+        a.out_ptr = c->d_out_ptr;
+        a.in_ptr = c->d_in_ptr;
+        a.row_src = c->d_val;
+        a.row_sign = c->d_val_alt;
+        a.row_tgt = reinterpret_cast<int32_t *>(c->d_key32);
+        a.row_k = reinterpret_cast<int32_t *>(c->d_key32_alt);
+        a.in_syn = c->d_in_syn;
+        a.retract_ax = retract_ax;
+        a.retract_de = retract_de;
+        a.vac_ax = vac_ax;
+        a.vac_de = vac_de;
+        a.need_ax = c->d_need_ax;
+        a.need_de = c->d_need_de;
+        a.prio_ax = c->d_prio_ax;
+        a.prio_de = c->d_prio_de;
+        a.sel_ax = c->d_sel_ax;
+        a.sel_de = c->d_sel_de;
+        a.broken = c->d_i64 + I64_BROKEN;
+        delete_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+            a, store_args(c, p.seed, (uint32_t)p.step));
+        note_launch();
+        c->canonical = false; // as below
+        return cudaGetLastError();
+    }
     if (!c->canonical && (e = canonicalise_store(c, st))) return e;
     delete_needs_kernel<<<gn, 256, 0, st>>>(n, retract_ax, retract_de, vac_ax, vac_de,
                                             c->d_out_ptr, c->d_in_ptr, c->d_need_ax,
                                             c->d_need_de);
     note_launch();
     delete_prio_kernel<<<gs, 256, 0, st>>>(dm, c->d_syn_src, c->d_in_syn, c->d_syn_tgt,
-                                           c->d_out_ptr, c->d_in_ptr, c->d_prio_ax, c->d_prio_de,
+                                           c->d_out_ptr, c->d_in_ptr, c->d_need_ax,
+                                           c->d_need_de, c->d_prio_ax, c->d_prio_de,
                                            c->d_sel_ax, c->d_sel_de, p.seed, (uint32_t)p.step);
     note_launch();
     delete_select_kernel<<<gn, 256, 0, st>>>(n, c->d_out_ptr, c->d_need_ax, c->d_prio_ax, nullptr,
@@ -591,6 +943,13 @@ cudaError_t merge_type(relearn_ctx *c, const int32_t *part, const uint8_t *type,
 cudaError_t deliver_spikes(relearn_ctx *c, const uint8_t *spiked, int32_t *input,
                            cudaStream_t st)
 {
+    if (small_network(c)) {
+        deliver_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
+            c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, spiked, nullptr, 0, 0, c->n,
+            input);
+        note_launch();
+        return cudaGetLastError();
+    }
     cudaError_t e;
     if ((e = cudaMemsetAsync(input, 0, c->n * sizeof(int32_t), st))) return e;
     spikes_kernel<<<grid_for(c->max_synapses, 256, c->num_sms), 256, 0, st>>>(
