@@ -829,30 +829,39 @@ __device__ __forceinline__ int warp_sum_i(int v)
 // block starts: lane k sums the ranges ord[k * per .. (k + 1) * per) on top of
 // start[k] (see split_walk).
 struct SplitLists {
-    double *start;                          // [32] prefix before each lane's block
-    int32_t *give_b, *give_e, *give_next;   // [32] hand-over slots of one step
-    int32_t *b;                             // [cap] first node of each range
-    float *part;                            // [cap] its compensated partial sum
-    int16_t *next;                          // [cap] the range after it in pre-order
-    int16_t *ord;                           // [cap] ranges in pre-order
+    double *start; // [32] prefix before each lane's block
+    int4 *give;    // [32] hand-over slots of one step: first node, end, next range
+    int2 *rec;     // [cap] range r: its compensated partial sum (float bits), and in two
+                   // halves the range after it in pre-order and the r-th range in pre-order
+    int32_t *b;    // [cap] first node of each range
     int cap;
+
+    __device__ __forceinline__ void done(int r, float part, int32_t next) const
+    {
+        rec[r] = make_int2(__float_as_int(part), next & 0xffff);
+    }
+    __device__ __forceinline__ float part(int r) const { return __int_as_float(rec[r].x); }
+    __device__ __forceinline__ int next(int r) const
+    {
+        return reinterpret_cast<const int16_t *>(&rec[r].y)[0];
+    }
+    __device__ __forceinline__ int16_t &ord(int r) const
+    {
+        return reinterpret_cast<int16_t *>(&rec[r].y)[1];
+    }
 };
 __host__ __device__ constexpr size_t split_warp_bytes(int cap)
 {
-    return 32 * sizeof(double) + 3 * 32 * sizeof(int32_t) + (size_t)cap * 12;
+    return 32 * sizeof(double) + 32 * sizeof(int4) + (size_t)cap * 12; // a multiple of 16
 }
 __device__ __forceinline__ SplitLists split_lists(unsigned char *raw, int w, int cap)
 {
-    unsigned char *base = raw + (size_t)w * split_warp_bytes(cap); // 8-byte aligned
+    unsigned char *base = raw + (size_t)w * split_warp_bytes(cap);
     SplitLists L;
     L.start = reinterpret_cast<double *>(base);
-    L.give_b = reinterpret_cast<int32_t *>(base + 32 * sizeof(double));
-    L.give_e = L.give_b + 32;
-    L.give_next = L.give_e + 32;
-    L.b = L.give_next + 32;
-    L.part = reinterpret_cast<float *>(L.b + cap);
-    L.next = reinterpret_cast<int16_t *>(L.part + cap);
-    L.ord = L.next + cap;
+    L.give = reinterpret_cast<int4 *>(base + 32 * sizeof(double));
+    L.rec = reinterpret_cast<int2 *>(L.give + 32);
+    L.b = reinterpret_cast<int32_t *>(L.rec + cap);
     L.cap = cap;
     return L;
 }
@@ -864,14 +873,19 @@ __device__ __forceinline__ int split_locate(const SplitLists &L, int n_rec, doub
 {
     const int per = (n_rec + 31) >> 5;
     const int nb = (n_rec + per - 1) / per; // non-empty blocks
-    int k = 0;
-    for (int j = 1; j < nb; ++j)
-        if (L.start[j] <= tgt) k = j;
+    int k = 0; // the last block that starts at or before tgt (the starts do not decrease)
+    for (int hi = nb - 1; k < hi;) {
+        const int mid = (k + hi + 1) >> 1;
+        if (L.start[mid] <= tgt)
+            k = mid;
+        else
+            hi = mid - 1;
+    }
     const int q0 = k * per, q1 = min(q0 + per, n_rec);
     double run = 0.0;
     for (int q = q0; q < q1; ++q) {
         const double before = L.start[k] + run;
-        run += (double)L.part[L.ord[q]];
+        run += (double)L.part(L.ord(q));
         if (L.start[k] + run > tgt || q == q1 - 1) {
             base = before;
             return q;
@@ -885,6 +899,7 @@ __device__ __forceinline__ int split_locate(const SplitLists &L, int n_rec, doub
 // calls it. Returns the number of ranges and S (every lane); own (this lane's
 // evaluations), dmin2 (nearest candidate this lane met) and steps (walk steps,
 // lane 0) accumulate.
+template <bool kCount>
 __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, int32_t root,
                                           int32_t root_end, float3 x, int32_t self_node,
                                           uint32_t thr0, float k2, float k2sh, int32_t &own,
@@ -897,8 +912,7 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
     bool busy = false;
     if (lane == 0) {
         L.b[0] = root + 1;
-        L.part[0] = 0.0f;
-        L.next[0] = -1;
+        L.done(0, 0.0f, -1);
         rid = 0;
         p = root + 1;
         e = root_end;
@@ -916,7 +930,7 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
             const float d2 = dist2(x, g);
             const bool has = g.w > 0.0f;
             const bool acc = has && (__float_as_uint(d2) + (uint32_t)t.y > thr0);
-            own += has ? 1 : 0;
+            if (kCount) own += has ? 1 : 0;
             if (acc && p != self_node) {
                 kahan_add(cum, comp, attraction(g.w, d2, k2, k2sh));
                 dmin2 = fminf(dmin2, d2);
@@ -929,32 +943,30 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
                 p = max(t.x, p + 1);
             }
             if (p >= e) { // range done
-                L.part[rid] = __fsub_rn(cum, comp);
-                L.next[rid] = (int16_t)rnext;
+                L.done(rid, __fsub_rn(cum, comp), rnext);
                 busy = false;
                 split = false;
             }
         }
         const uint32_t idle = __ballot_sync(0xffffffffu, !busy);
         if (idle == 0xffffffffu) break;
-        steps += lane == 0 ? 1 : 0;
+        if (kCount) steps += lane == 0 ? 1 : 0;
         const uint32_t spl = __ballot_sync(0xffffffffu, split);
         const int give = min(min(__popc(idle), __popc(spl)), L.cap - n_rec);
         if (give > 0) { // warp-uniform: the r-th splitting lane gives to the r-th idle lane
             const int rs = __popc(spl & lt), ri = __popc(idle & lt);
             if (split && rs < give) {
-                L.give_b[rs] = rest;
-                L.give_e[rs] = e;
-                L.give_next[rs] = rnext;
+                L.give[rs] = make_int4(rest, e, rnext, 0);
                 e = rest;
                 rnext = n_rec + rs;
             }
             __syncwarp();
             if (!busy && ri < give) {
                 rid = n_rec + ri;
-                p = L.give_b[ri];
-                e = L.give_e[ri];
-                rnext = L.give_next[ri];
+                const int4 v = L.give[ri];
+                p = v.x;
+                e = v.y;
+                rnext = v.z;
                 L.b[rid] = p;
                 cum = 0.0f;
                 comp = 0.0f;
@@ -969,8 +981,9 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
     if (lane == 0) {
         int r = 0;
         for (int pos = 0; pos < n_rec; ++pos) { // the links reach every range once
-            L.ord[pos] = (int16_t)(r >= 0 ? r : 0);
-            if (r >= 0) r = L.next[r];
+            const int nx = r >= 0 ? L.next(r) : -1;
+            L.ord(pos) = (int16_t)(r >= 0 ? r : 0);
+            r = nx;
         }
     }
     __syncwarp();
@@ -981,7 +994,7 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
     const int per = (n_rec + 31) >> 5;
     const int q0 = min(lane * per, n_rec), q1 = min(q0 + per, n_rec);
     double blk = 0.0;
-    for (int q = q0; q < q1; ++q) blk += (double)L.part[L.ord[q]];
+    for (int q = q0; q < q1; ++q) blk += (double)L.part(L.ord(q));
     double start = __shfl_up_sync(0xffffffffu, blk, 1);
     if (lane == 0) start = 0.0;
 #pragma unroll
@@ -996,7 +1009,7 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
     return n_rec;
 }
 
-template <bool kBatched>
+template <bool kBatched, bool kCount>
 __global__ void __launch_bounds__(256) bh_split_kernel(SearchArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_raw[]; // 8 x split_warp_bytes(cap)
@@ -1034,7 +1047,7 @@ __global__ void __launch_bounds__(256) bh_split_kernel(SearchArgs a)
         for (int attempt = 0; attempt < 2; ++attempt) {
             float dmin2 = __int_as_float(0x7f800000);
             own = 0;
-            n_rec = split_walk(a, L, root, root_end, x, self_node, thr0, k2, k2sh, own, dmin2,
+            n_rec = split_walk<kCount>(a, L, root, root_end, x, self_node, thr0, k2, k2sh, own, dmin2,
                                my_steps, S);
             if (!(S < (double)kTiny)) break;
             // every term underflowed: redo with the exponents shifted by the nearest d^2
@@ -1044,8 +1057,10 @@ __global__ void __launch_bounds__(256) bh_split_kernel(SearchArgs a)
             k2sh = __fmul_rn(k2, dmin2);
             __syncwarp();
         }
-        own = warp_sum_i(own);
-        if (lane == 0) my_evals += own;
+        if (kCount) {
+            own = warp_sum_i(own);
+            if (lane == 0) my_evals += own;
+        }
 
         // ---- draws: the source's searches, one per lane
         const int32_t i = a.perm[s];
@@ -1062,8 +1077,8 @@ __global__ void __launch_bounds__(256) bh_split_kernel(SearchArgs a)
                 const double tgt = (double)u * 2.3283064365386963e-10 * S;
                 double base;
                 const int lo = split_locate(L, n_rec, tgt, base); // range holding u * S
-                const int32_t rb = L.b[L.ord[lo]];
-                const int32_t re = lo + 1 < n_rec ? L.b[L.ord[lo + 1]] : root_end;
+                const int32_t rb = L.b[L.ord(lo)];
+                const int32_t re = lo + 1 < n_rec ? L.b[L.ord(lo + 1)] : root_end;
                 const int32_t k = range_find(a.nodes, rb, re, x, self_node, thr0, k2, k2sh,
                                              (float)(tgt - base));
                 result = restart_chain(a, k, x, self_node, thr0, k2, i, e, evals, draws,
@@ -1080,16 +1095,18 @@ __global__ void __launch_bounds__(256) bh_split_kernel(SearchArgs a)
         }
         __syncwarp(); // the lists are reused by the next source
     }
-    for (int off = 16; off; off >>= 1) {
-        my_evals += __shfl_xor_sync(0xffffffffu, my_evals, off);
-        my_steps += __shfl_xor_sync(0xffffffffu, my_steps, off);
+    if constexpr (kCount) {
+        for (int off = 16; off; off >>= 1) {
+            my_evals += __shfl_xor_sync(0xffffffffu, my_evals, off);
+            my_steps += __shfl_xor_sync(0xffffffffu, my_steps, off);
+        }
+        if (lane == 0 && my_evals)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.evals_total),
+                      (unsigned long long)my_evals);
+        if (lane == 0 && my_steps)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.steps_total),
+                      (unsigned long long)my_steps);
     }
-    if (a.count && lane == 0 && my_evals)
-        atomicAdd(reinterpret_cast<unsigned long long *>(a.evals_total),
-                  (unsigned long long)my_evals);
-    if (a.count && lane == 0 && my_steps)
-        atomicAdd(reinterpret_cast<unsigned long long *>(a.steps_total),
-                  (unsigned long long)my_steps);
 }
 
 // Deferred restarts, one thread per queued search, in the order of their drawn
@@ -1256,7 +1273,10 @@ cudaError_t search_run(relearn_ctx *c, const relearn_params &p, const int32_t *v
                                                 : bh_search_kernel<true, false>)
                                      : (a.count ? bh_search_kernel<false, true>
                                                 : bh_search_kernel<false, false>);
-    void (*split)(SearchArgs) = a.net ? bh_split_kernel<true> : bh_split_kernel<false>;
+    void (*split)(SearchArgs) = a.net ? (a.count ? bh_split_kernel<true, true>
+                                                 : bh_split_kernel<true, false>)
+                                      : (a.count ? bh_split_kernel<false, true>
+                                                 : bh_split_kernel<false, false>);
     // resident blocks per SM of both kernels, queried once per context, kernel pair and
     // split capacity
     a.split_cap = split_capacity(p.theta);
@@ -1265,14 +1285,16 @@ cudaError_t search_run(relearn_ctx *c, const relearn_params &p, const int32_t *v
     int &occ_split = c->split_occ[a.net ? 1 : 0][a.split_cap / 32];
     if (occ[0] == 0) {
         int per_sm = 0;
-        // both counting variants have the same launch bounds
+        // (of both kernels the counting variants are launched alike)
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                  &per_sm, a.net ? bh_search_kernel<true, false> : bh_search_kernel<false, false>,
                  256, 0)))
             return e;
-        if ((e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(8 * split_warp_bytes(kSplitMaxCap)))))
-            return e;
+        for (auto k : {bh_split_kernel<false, false>, bh_split_kernel<false, true>,
+                       bh_split_kernel<true, false>, bh_split_kernel<true, true>})
+            if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(8 * split_warp_bytes(kSplitMaxCap)))))
+                return e;
         occ[0] = per_sm < 1 ? 1 : per_sm;
     }
     if (occ_split == 0) {
