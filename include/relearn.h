@@ -383,7 +383,7 @@ relearn_status relearn_peak_probe(int32_t kind, int64_t iters, float *buf, int64
  *   codes        device uint32[n], out: the codes in ascending order.
  *   perm         device int32[n], out: perm[k] = id of the neuron with the k-th code
  *                (ties by id), the same order relearn_get_tree reports.
- * The sort's scratch is one static device array of about 8.5 MB per GPU, held until the
+ * The sort's scratch is one static device array of about 9 MB per GPU, held until the
  * process exits. Every call looks up that array's device address on the current device
  * (a lookup, no allocation); the first call on each device also reads its SM count and
  * may make the driver load this library's kernels there, so make that first call before

@@ -72,6 +72,7 @@ void free_all(relearn_ctx *c)
         (void **)&c->d_status,   (void **)&c->d_i64,        (void **)&c->d_i32,
         (void **)&c->d_geom,     (void **)&c->d_sc,         (void **)&c->d_codes,
         (void **)&c->d_off,      (void **)&c->d_ord,        (void **)&c->d_root,
+        (void **)&c->d_box,
         (void **)&c->d_net,      (void **)&c->d_nkey,       (void **)&c->d_nkey_alt,
         (void **)&c->d_lstate,   (void **)&c->d_lsum,       (void **)&c->d_fam,
         (void **)&c->d_rq_key,   (void **)&c->d_rq_key_alt, (void **)&c->d_rq_val,
@@ -202,6 +203,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(d_sc, NB);
     A(d_off, NB + 1);
     A(d_ord, 6 * NB);
+    A(d_box, 2048);
     A(d_root, NB);
     A(d_lstate, N);
     A(d_fam, M + 8); // walks read whole families of eight
@@ -266,10 +268,9 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(d_need_de, N);
     A(d_keep, S + 1);
     const int64_t sort_blocks = sort_blocks_needed(std::max({N, S, QC}));
-    A(sort.hist, 256 * sort_blocks);
+    A(sort.hist, sort_scratch_words(sort_blocks));
     int64_t scan_blocks = std::max({scan_blocks_needed(N + 1), scan_blocks_needed(QC),
-                                    scan_blocks_needed(S), scan_blocks_needed(256 * sort_blocks),
-                                    scan_blocks_needed(M)});
+                                    scan_blocks_needed(S), scan_blocks_needed(M)});
     A(scan.block_sums, 4 * scan_blocks); // a pair scan keeps two sums per tile
     A(scan.flags, scan_blocks + 3);
 #undef A
@@ -280,6 +281,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
         c->scan.status = c->d_status;
         c->scan.grid_cap = scan_grid_cap(c->num_sms);
         c->sort.max_blocks = sort_blocks;
+        c->sort.num_sms = c->num_sms;
         c->sort.scan = c->scan;
         for (cudaEvent_t &ev : c->ev)
             if (e == cudaSuccess) e = cudaEventCreate(&ev);
@@ -290,6 +292,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_off, (NB + 1) * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->off_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMemset(c->d_box, 0, sizeof(uint32_t));
     if (e == cudaSuccess)
         e = cudaMemset(c->scan.flags, 0, (c->scan.max_blocks + 3) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_i64, 0, 16 * sizeof(int64_t));

@@ -1,7 +1,10 @@
 // Host-side internals of librelearn: the context and the kernel launchers that
 // the translation units share. Not installed; the public ABI is relearn.h.
 #pragma once
+#include <algorithm>
 #include <cstdint>
+#include <utility>
+
 #include <cuda_runtime.h>
 
 #include "../../include/relearn.h"
@@ -20,11 +23,12 @@ struct ScanScratch {
     int64_t grid_cap = 1 << 30;    // blocks a scan launches at most (the resident ones)
 };
 
-// Scratch of the LSD radix sort (per-block digit histograms, digit-major).
+// Scratch of the LSD radix sort.
 struct SortScratch {
-    int32_t *hist = nullptr;      // [256 * max_blocks]
+    int32_t *hist = nullptr; // [sort_scratch_words(max_blocks)]
     int64_t max_blocks = 0;
-    ScanScratch scan;
+    int num_sms = 1;
+    ScanScratch scan; // (its status word)
 };
 
 // Per-build geometry, device resident.
@@ -74,6 +78,7 @@ struct relearn_ctx {
     int64_t *h_off = nullptr;     // [max_nets + 1] pinned staging of the offsets
     cudaEvent_t off_ev = nullptr; // the last copy out of h_off
     uint32_t *d_ord = nullptr;    // [6 * max_nets] bounding boxes (ordered-int min, max)
+    uint32_t *d_box = nullptr;    // [2048] one network: a count and the blocks' boxes
     int32_t *d_root = nullptr;    // [max_nets] root node of each network
     int32_t *d_net = nullptr;     // [n] network of each Morton position (max_nets > 1)
     uint64_t *d_nkey = nullptr, *d_nkey_alt = nullptr; // [n] (network, code) sort keys
@@ -153,7 +158,7 @@ namespace rl {
 // Whether a context's passes over its neurons and synapses run as one cluster kernel each
 // (cluster.cuh): by its sizes and capacities, since the counts of searches and synapses
 // are known on the device only.
-constexpr int64_t kSmallN = 40960, kSmallItems = 8 * kSmallN;
+constexpr int64_t kSmallN = 40960, kSmallItems = 8 * kSmallN, kSmallBuildN = 32768;
 inline bool small_network(const relearn_ctx *c)
 {
     return c->n <= kSmallN && c->max_searches <= kSmallItems && c->max_synapses <= kSmallItems;
@@ -185,13 +190,18 @@ cudaError_t fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t st);
 // sort.cu -------------------------------------------------------------------
 // Stable LSD radix sort of (key, val) on bits [0, end_bit). Returns the buffer
 // index holding the result (0: keys/vals, 1: the *_alt buffers) through *which.
+// counted: sort_clear_u32 was called for max_n elements before, and a kernel since has
+// added each key's digits p (8 bits each) to sort_counts()[256 * p + digit].
 cudaError_t radix_sort_u32(uint32_t *keys, uint32_t *keys_alt, int32_t *vals, int32_t *vals_alt,
                            int64_t max_n, const int32_t *d_count, int end_bit, SortScratch &s,
-                           cudaStream_t st, int *which);
+                           cudaStream_t st, int *which, bool counted = false);
+cudaError_t sort_clear_u32(int64_t n, SortScratch &s, cudaStream_t st);
+uint32_t *sort_counts(SortScratch &s);
 cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int32_t *vals, int32_t *vals_alt,
                            int64_t max_n, const int32_t *d_count, int end_bit, SortScratch &s,
                            cudaStream_t st, int *which);
 int64_t sort_blocks_needed(int64_t max_n);
+int64_t sort_scratch_words(int64_t blocks);
 
 // Launch attributes of each file's cluster kernels on the current device.
 cudaError_t octree_init();
