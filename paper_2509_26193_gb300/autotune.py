@@ -3,8 +3,8 @@
 The search kernel walks the octree with unions of source neurons that are adjacent
 in Morton order (``search_group`` in relearn_params). By default each warp's 32
 sources are cut into pieces wherever two neighbours do not share a cell of some
-cut depth, and each piece walks one union; the cut depth follows the share of
-neurons that search. A fixed width (32, 8, or every lane alone) or another cut depth
+cut depth, and each piece walks one union; the cut depth is chosen per warp from
+how many pieces it makes. A fixed width (32, 8, or every lane alone) or another cut depth
 can be forced. The best choice depends on the workload (cluster sizes, density,
 sigma relative to the domain). Results never depend on the choice, only the time
 does, so the tuner simply times each candidate on the caller's own update and keeps

@@ -190,6 +190,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     c->max_synapses = max_synapses;
     c->max_searches = max_searches ? max_searches : std::min<int64_t>(8 * max_neurons, 0x7ffffff0);
     c->max_nodes = 2 * max_neurons + 1;
+    if (max_networks > 1) c->max_nodes += kPad * (int64_t)max_networks; // walk sentinels
     const int64_t N = max_neurons, S = max_synapses, QC = c->max_searches, M = c->max_nodes;
     std::vector<void *> owned;
     cudaError_t e = cudaSuccess;
@@ -704,6 +705,8 @@ relearn_status relearn_get_tree(relearn_ctx *c, int64_t capacity, int64_t *num_n
     relearn_status s = sync(c);
     int64_t m = 0;
     CK(cudaMemcpy(&m, c->d_i64 + I64_NODES, sizeof(m), cudaMemcpyDeviceToHost), "copy");
+    const int64_t stored = m;
+    if (c->num_nets > 1) m -= kPad * (int64_t)c->num_nets; // each network's walk sentinels
     *num_nodes = m;
     const int64_t n = c->n;
     std::vector<int32_t> hp;
@@ -714,18 +717,21 @@ relearn_status relearn_get_tree(relearn_ctx *c, int64_t capacity, int64_t *num_n
     }
     if (depth || first || size || is_leaf || neuron || count || cx || cy || cz) {
         if (capacity < m) return fail(c, RELEARN_ERR_INVALID_ARG, "get_tree: capacity");
-        std::vector<Node> h(m);
-        std::vector<int32_t> par(m);
-        CK(cudaMemcpy(h.data(), c->d_nodes, m * sizeof(Node), cudaMemcpyDeviceToHost), "copy");
-        CK(cudaMemcpy(par.data(), c->d_parent, m * sizeof(int32_t), cudaMemcpyDeviceToHost),
+        std::vector<Node> h(stored);
+        std::vector<int32_t> par(stored);
+        CK(cudaMemcpy(h.data(), c->d_nodes, stored * sizeof(Node), cudaMemcpyDeviceToHost), "copy");
+        CK(cudaMemcpy(par.data(), c->d_parent, stored * sizeof(int32_t), cudaMemcpyDeviceToHost),
            "copy");
-        for (int64_t v = 0; v < m; ++v) {
-            const Node &nd = h[v];
+        for (int64_t u = 0, v = -1; u < stored; ++u) {
+            const Node &nd = h[u];
             const bool leaf = node_is_leaf(nd.t.shift);
+            // a sentinel: at depth 0 and without a subtree (a root has at least its leaf)
+            if (nd.t.shift == 0u && nd.t.escape == u + 1) continue;
+            ++v;
             const int32_t f = nd.t.neuron;
-            const int32_t fe = nd.t.escape < m ? h[nd.t.escape].t.neuron : (int32_t)n;
+            const int32_t fe = nd.t.escape < stored ? h[nd.t.escape].t.neuron : (int32_t)n;
             // a leaf sits one level below its parent (depth 11 inside a bucket)
-            const int dep = leaf ? (par[v] >= 0 ? depth_of(h[par[v]].t.shift) + 1 : 0)
+            const int dep = leaf ? (par[u] >= 0 ? depth_of(h[par[u]].t.shift) + 1 : 0)
                                  : depth_of(nd.t.shift);
             if (depth) depth[v] = dep;
             if (first) first[v] = f;

@@ -413,12 +413,18 @@ __global__ void topo_pairs_kernel(const uint32_t *__restrict__ codes,
     }
 }
 
+// Nodes that start at each position: its cells and its leaf; in a batch also the kPad
+// sentinels after a network's last leaf.
 __global__ void topo_count_kernel(const uint32_t *__restrict__ mask, int64_t n,
-                                  int32_t *__restrict__ cnt)
+                                  const int32_t *__restrict__ net,
+                                  const int64_t *__restrict__ off, int32_t *__restrict__ cnt)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        cnt[i] = i < n ? __popc(mask[i]) + 1 : 0;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int32_t c = i < n ? __popc(mask[i]) + 1 : 0;
+        if (net && i < n && i + 1 == off[net[i] + 1]) c += kPad;
+        cnt[i] = c;
+    }
 }
 
 // Parent of a node whose shallower ancestors do not start at position i: the
@@ -442,9 +448,10 @@ struct TopoOut {
 
 // The nodes that start at position i of a network at [lo, hi): its cells in m = mask[i],
 // outermost first, then the leaf of position i.
-__device__ __forceinline__ void topo_emit(int64_t i, int64_t lo, int64_t hi, const uint32_t *codes,
-                                          const uint32_t *mask, const int32_t *base,
-                                          const TopoOut &o)
+// pad: sentinels between the network's last node and the next network's root.
+__device__ __forceinline__ void topo_emit(int64_t i, int64_t lo, int64_t hi, int pad,
+                                          const uint32_t *codes, const uint32_t *mask,
+                                          const int32_t *base, const TopoOut &o)
 {
     const uint32_t m = mask[i];
     const int32_t b = base[i];
@@ -464,7 +471,7 @@ __device__ __forceinline__ void topo_emit(int64_t i, int64_t lo, int64_t hi, con
         }
         Node nd;
         nd.g = NodeGeo{0.f, 0.f, 0.f, 0.f};
-        nd.t = NodeTopo{base[R + 1], (uint32_t)d << 24, (int32_t)i, 0};
+        nd.t = NodeTopo{base[R + 1] - (R + 1 == hi ? pad : 0), (uint32_t)d << 24, (int32_t)i, 0};
         o.nodes[v] = nd;
         o.parent[v] = par;
         o.nsize[v] = (int32_t)(R - i + 1);
@@ -487,12 +494,12 @@ __device__ __forceinline__ void topo_emit(int64_t i, int64_t lo, int64_t hi, con
     o.leaf_of[i] = v;
 }
 
-// Nodes m .. m + 2, past the last one (m nodes), are sentinels for walks that step past the
-// end: no count, escape = next node.
-__device__ __forceinline__ void sentinel(Node *nodes, int64_t v)
+// Sentinels for walks that step past the end of a network's tree (kPad nodes): no count,
+// escape = next node, first position = the end of the network's.
+__device__ __forceinline__ void sentinel(Node *nodes, int64_t v, int64_t end)
 {
     nodes[v].g = NodeGeo{0.f, 0.f, 0.f, 0.f};
-    nodes[v].t = NodeTopo{(int32_t)(v + 1), 0u, -1, 0};
+    nodes[v].t = NodeTopo{(int32_t)(v + 1), 0u, (int32_t)end, 0};
 }
 
 __global__ void topo_emit_kernel(const uint32_t *__restrict__ codes,
@@ -502,13 +509,22 @@ __global__ void topo_emit_kernel(const uint32_t *__restrict__ codes,
                                  const int32_t *__restrict__ base, TopoOut o,
                                  int32_t *__restrict__ root, const int64_t *d_num_nodes)
 {
-    if (blockIdx.x == 0 && threadIdx.x < 3) sentinel(o.nodes, *d_num_nodes + threadIdx.x);
+    // past the last node (one network; in a batch every network's are part of the nodes)
+    if (blockIdx.x == 0 && threadIdx.x < kPad) sentinel(o.nodes, *d_num_nodes + threadIdx.x, n);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t nb = net_at(net, i);
         const int64_t lo = off[nb];
         if (i == lo) root[nb] = base[i]; // the first node at a network's first position
-        topo_emit(i, lo, off[nb + 1], codes, mask, base, o);
+        const int64_t hi = off[nb + 1];
+        topo_emit(i, lo, hi, net ? kPad : 0, codes, mask, base, o);
+        if (net && i + 1 == hi)
+            for (int k = 0; k < kPad; ++k) {
+                const int32_t v = base[i + 1] - kPad + k;
+                sentinel(o.nodes, v, hi);
+                o.parent[v] = -1;
+                o.nsize[v] = 0;
+            }
     }
 }
 
@@ -724,8 +740,9 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
         [&](int64_t i, cf::I32 prefix, cf::I32, cf::I32) { t.base[i] = prefix.v; });
     cf::sync();
     if (tid == 0) *t.d_num_nodes = m.v;
-    if (tid < 3) sentinel(t.o.nodes, m.v + tid);
-    for (int64_t i = tid; i < n; i += cf::kStride) topo_emit(i, 0, n, a.codes, t.mask, t.base, t.o);
+    if (tid < kPad) sentinel(t.o.nodes, m.v + tid, n);
+    for (int64_t i = tid; i < n; i += cf::kStride) 
+        topo_emit(i, 0, n, 0, a.codes, t.mask, t.base, t.o);
 }
 
 // Bottom-up update as prefix sums (Sec. III-B "Division of work": an inner node
@@ -1123,7 +1140,8 @@ cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, c
     note_launch();
     topo_pairs_kernel<<<gn, 256, 0, st>>>(c->d_codes, net, c->d_off, n, c->d_mask);
     note_launch();
-    topo_count_kernel<<<grid_for(n + 1, 256, c->num_sms), 256, 0, st>>>(c->d_mask, n, c->d_cnt);
+    topo_count_kernel<<<grid_for(n + 1, 256, c->num_sms), 256, 0, st>>>(c->d_mask, n, net,
+                                                                         c->d_off, c->d_cnt);
     note_launch();
     if ((e = scan_exclusive(c->d_cnt, c->d_base, n + 1, nullptr, c->d_i64 + I64_NODES, c->scan,
                             st)))

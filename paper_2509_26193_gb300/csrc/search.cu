@@ -50,20 +50,22 @@ constexpr int kCkStride = 128; // warp steps between checkpoints (times 2^k once
 constexpr int kMaxCk = 128;    // checkpoints kept per lane
 constexpr float kTiny = 8.673617e-19f; // 2^-60
 // Walks per warp (see bh_search_kernel): the warp's 32 sources are cut into pieces at
-// the boundaries of cells of some depth, and each piece walks one union. With one
-// network the warp's pieces step in blocks of four like a single union, so fine cuts
-// cost little: depth kCutSingle (cells of 1/64 of the domain's edge). Sweep on the
-// 2^20-neuron clustered network (first three updates, 86 / 40 / 15 % of the neurons
-// searching): depth 2 6.85 / 4.12 / 2.74 ms, depth 4 6.87 / 3.78 / 2.27, depth 5
-// 6.83 / 3.78 / 2.16, depth 6 6.77 / 3.78 / 2.16, depth 7 7.24 / 4.10 / 2.81,
-// depth 10 13.65 / 6.84 / 4.05. With several networks (pieces stepped one step per
-// test) the cut follows the share of neurons searching: the more search, the closer
-// consecutive sources are, and the coarser the cut can be before a union spans
-// sources too far apart: depth 2 when at least kDenseTenths / 10 of the neurons
-// search, depth 3 from kMidTenths / 10, else depth 4 (a batch of 256 uniform
-// networks, 86 % searching: depth 2 234.9 ms, depth 4 274.2 ms).
-constexpr int kCutSingle = 6;
-constexpr int kCutDense = 2, kCutMid = 3, kCutSparse = 4, kDenseTenths = 6, kMidTenths = 3;
+// the boundaries of cells of some depth, and each piece walks one union: finer pieces
+// make shorter walks, but every piece reads its own node at each step. The depth is
+// chosen per warp: the deepest one, up to kMaxCutDepth, that leaves at most kMaxCuts cuts
+// (four sources a piece; one depth for every warp suits one density: depth 6 is the best
+// in the 2^20 clusters and the 2^22 slab, depth 5 in a 2^20 cube). Search of the first
+// updates, ms, one depth 6 (a batch: 2) -> at most 2 / 4 / 7 / 10 / 15 cuts: 2^20 cube
+// 6.72 + 4.00 -> 6.35 + 3.51 / 6.34 + 3.28 / 6.33 + 3.30 / 6.67 + 3.31 / 6.74 + 3.60; 2^22
+// slab 52.0 + 24.0 -> 55.2 + 25.5 / 52.4 + 25.2 / 52.0 + 23.8 / 52.1 + 23.7 / 55.5 + 24.1;
+// 300,007 clustered neurons at theta 0.2 4.92 + 3.67 -> 4.68 + 3.64 with 7; 2^20 clusters
+// 6.51 + 3.65 -> 6.56 + 3.57 / 6.63 + 3.64 / 6.64 + 3.59 / 6.75 + 3.62 / 7.40 + 3.81;
+// batch of 64 networks 14.5 -> 11.2 with 7 (most of it the blocks of four steps, which a
+// batch takes too since every network has its own sentinels). Updates with at most
+// kFewSources sources per resident warp wait on their longest walks rather than on the
+// reads of many pieces: kMaxCutsFew (third update of the cube 2.50 -> 2.06 with 7, 1.77
+// with 11; with 11 for 27 sources per warp 4.93 instead of 4.70 ms).
+constexpr int kMaxCutDepth = 8, kMaxCuts = 7, kMaxCutsFew = 11, kFewSources = 20;
 // The default also looks at how many sources the update has, per resident warp of
 // the union kernel (W = 9,728 on 152 SMs at 8 blocks per SM; the sweeps below were
 // taken at 6 blocks, W = 7,296, and the threshold rechecked at 8). Per-update sweeps
@@ -229,7 +231,6 @@ struct SearchArgs {
     uint32_t step;
     int forced_group; // 0 = choose per warp; 1, 8, 16, 32 = union width; 2 = split
     int spread_depth;  // cut depth of union pieces (-1: the default by source density)
-    int64_t n_total;   // neurons of all networks
     int32_t split_below; // with forced_group 0: split kernel for at most this many sources
     int split_cap;       // ranges per source in the split kernel (split_capacity)
     // deferred restarts (RELEARN_FLAG_REGROUP): searches whose first draw is an inner
@@ -505,6 +506,7 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
         thr0 = __ldg(&a.sc->thr0);
         k2 = __ldg(&a.sc->k2);
     }
+    const int max_cuts = A <= (int32_t)gridDim.x * 8 * kFewSources ? kMaxCutsFew : kMaxCuts;
     int32_t ckp[kMaxCk];
     float ckc[kMaxCk];  // compensated running sum at each checkpoint
     float ckk[kMaxCk];  // its compensation term
@@ -549,17 +551,18 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
             uint32_t code = live ? a.codes[s] : 0u;
             code = __shfl_sync(0xffffffffu, code, live ? lane : last);
             const uint32_t nxt = __shfl_down_sync(0xffffffffu, code, 1);
-            const int depth = a.spread_depth >= 0                          ? a.spread_depth
-                              : !kBatched                                   ? kCutSingle
-                              : (int64_t)A * 10 >= kDenseTenths * a.n_total ? kCutDense
-                              : (int64_t)A * 10 >= kMidTenths * a.n_total   ? kCutMid
-                                                                            : kCutSparse;
-            bool cut = lane < 31 && morton_common_digits(code, nxt) < depth;
+            // the depth of the cell this lane's source shares with the next one (-1: they
+            // are in different networks)
+            int shared = lane < 31 ? morton_common_digits(code, nxt) : kMaxDepth;
             if constexpr (kBatched) {
                 const int32_t nn = __shfl_down_sync(0xffffffffu, net, 1);
-                cut = cut || (lane < 31 && nn != net);
+                if (lane < 31 && nn != net) shared = -1;
             }
-            const uint32_t cuts = __ballot_sync(0xffffffffu, cut); // bit i: cut after lane i
+            int depth = a.spread_depth >= 0 ? a.spread_depth : kMaxCutDepth;
+            uint32_t cuts = __ballot_sync(0xffffffffu, shared < depth); // bit i: cut after lane i
+            if (a.spread_depth < 0)
+                while (depth > 0 && __popc(cuts) > max_cuts)
+                    cuts = __ballot_sync(0xffffffffu, shared < --depth);
             const uint32_t below = cuts & ((1u << lane) - 1u);
             seg_first = below ? 32 - __clz(below) : 0;
             const uint32_t from = cuts >> lane;
@@ -613,20 +616,12 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
                     checkpoint(max(p, skip));
                     const int32_t p_blk = p;
                     int k = 0;
-                    if constexpr (!kBatched) {
-                        // four steps per test: nodes root_end .. root_end + 2 are
-                        // sentinels (no count, escape = next node), so steps past the
-                        // end change nothing
+                    // four steps per test: nodes root_end .. root_end + 2 are sentinels
+                    // (no count, escape = next node), so steps past the end change nothing
 #pragma unroll 1
-                        for (; k < kCkStride && p < root_end; k += 4) {
+                    for (; k < kCkStride && p < root_end; k += 4) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                union_step<kCount>(a.nodes, p, skip, cum, comp, own, x,
-                                                   self_node, thr0, k2, k2sh);
-                        }
-                    } else {
-#pragma unroll 1
-                        for (; k < kCkStride && p < root_end; ++k)
+                        for (int u = 0; u < 4; ++u)
                             union_step<kCount>(a.nodes, p, skip, cum, comp, own, x, self_node,
                                                thr0, k2, k2sh);
                     }
@@ -634,7 +629,7 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
                     if (p <= p_blk) break; // no progress: only a malformed tree
                 }
                 if (p > root_end) steps -= p - root_end; // the sentinels' steps
-            } else if constexpr (!kBatched) {
+            } else {
                 // several walks per warp (lane groups gmask) in the same blocks of four
                 // steps per test: a group that has finished parks on the sentinel at
                 // root_end (no count; its escape is clamped back to root_end)
@@ -655,28 +650,6 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
                     if (__any_sync(0xffffffffu, p < root_end && p <= p_blk)) break;
                 }
                 steps = gst;
-            } else {
-                while (__any_sync(0xffffffffu, p < root_end)) {
-                    const bool run = p < root_end; // uniform within the group
-                    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-                    int2 t = make_int2(p + 1, 0);
-                    if (run) {
-                        if ((steps & (kCkStride - 1)) == 0) checkpoint(max(p, skip));
-                        ++steps;
-                        load_node(&a.nodes[p], g, t);
-                    }
-                    const float d2 = dist2(x, g);
-                    const bool on = run && p >= skip && g.w > 0.0f;
-                    const bool pass = __float_as_uint(d2) + (uint32_t)t.y > thr0;
-                    if (kCount) own += on ? 1 : 0;
-                    if (on && pass) {
-                        skip = t.x;
-                        if (p != self_node)
-                            kahan_add(cum, comp, attraction(g.w, d2, k2, k2sh));
-                    }
-                    const uint32_t down = __ballot_sync(0xffffffffu, on && !pass) & gmask;
-                    if (run) p = down ? p + 1 : max(t.x, p + 1);
-                }
             }
             if (kCount && lane == seg_first) task_steps += steps; // one count per walk
             nck = ckst & 0xff;
@@ -1268,7 +1241,6 @@ cudaError_t search_run(relearn_ctx *c, const relearn_params &p, const int32_t *v
     a.forced_group = sg < 1000 ? (int)sg : 0;
     const bool depths = sg >= 1000 && sg < 3000;
     a.spread_depth = depths ? (int)((sg - 1000) / 100) : -1;
-    a.n_total = c->n;
     void (*kern)(SearchArgs) = a.net ? (a.count ? bh_search_kernel<true, true>
                                                 : bh_search_kernel<true, false>)
                                      : (a.count ? bh_search_kernel<false, true>
