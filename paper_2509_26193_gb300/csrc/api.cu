@@ -726,7 +726,7 @@ relearn_status relearn_get_tree(relearn_ctx *c, int64_t capacity, int64_t *num_n
             const Node &nd = h[u];
             const bool leaf = node_is_leaf(nd.t.shift);
             // a sentinel: at depth 0 and without a subtree (a root has at least its leaf)
-            if (nd.t.shift == 0u && nd.t.escape == u + 1) continue;
+            if (nd.t.shift == 0u && nd.t.escape == u) continue;
             ++v;
             const int32_t f = nd.t.neuron;
             const int32_t fe = nd.t.escape < stored ? h[nd.t.escape].t.neuron : (int32_t)n;

@@ -110,7 +110,7 @@ __device__ __forceinline__ void load_node(const Node *n, float4 &g, int2 &t)
 }
 
 constexpr int kMaxDepth = 10;
-constexpr int kPad = 3; // sentinel nodes after a tree (walks take four steps per bounds test)
+constexpr int kPad = 1; // sentinel nodes after a tree (walks take four steps per bounds test)
 
 
 // Number of leading octal digits (octree levels) two Morton codes share; 10 when equal.

@@ -494,12 +494,12 @@ __device__ __forceinline__ void topo_emit(int64_t i, int64_t lo, int64_t hi, int
     o.leaf_of[i] = v;
 }
 
-// Sentinels for walks that step past the end of a network's tree (kPad nodes): no count,
-// escape = next node, first position = the end of the network's.
+// The sentinel for walks that step on at the end of a network's tree: no count, escape =
+// the node itself (walks stay on it), first position = the network's end.
 __device__ __forceinline__ void sentinel(Node *nodes, int64_t v, int64_t end)
 {
     nodes[v].g = NodeGeo{0.f, 0.f, 0.f, 0.f};
-    nodes[v].t = NodeTopo{(int32_t)(v + 1), 0u, (int32_t)end, 0};
+    nodes[v].t = NodeTopo{(int32_t)v, 0u, (int32_t)end, 0};
 }
 
 __global__ void topo_emit_kernel(const uint32_t *__restrict__ codes,

@@ -46,8 +46,12 @@ namespace rl {
 
 namespace {
 
-constexpr int kCkStride = 128; // warp steps between checkpoints (times 2^k once the list fills)
-constexpr int kMaxCk = 128;    // checkpoints kept per lane
+// Warp steps between checkpoints (times 2^k once the list fills) and checkpoints kept per
+// lane: a draw walks half an interval on average. Steps between, ms of the first update's
+// search: 2^20 clusters 128 6.35, 64 6.02, 32 6.13; batch of 64 networks 10.8, 10.1, 10.0;
+// 2^22 slab 48.5, 48.4, 48.9 (with 192 instead of 128 checkpoints 47.8, clusters 5.99).
+constexpr int kCkStride = 64;
+constexpr int kMaxCk = 192;
 constexpr float kTiny = 8.673617e-19f; // 2^-60
 // Walks per warp (see bh_search_kernel): the warp's 32 sources are cut into pieces at
 // the boundaries of cells of some depth, and each piece walks one union: finer pieces
@@ -64,8 +68,10 @@ constexpr float kTiny = 8.673617e-19f; // 2^-60
 // batch takes too since every network has its own sentinels). Updates with at most
 // kFewSources sources per resident warp wait on their longest walks rather than on the
 // reads of many pieces: kMaxCutsFew (third update of the cube 2.50 -> 2.06 with 7, 1.77
-// with 11; with 11 for 27 sources per warp 4.93 instead of 4.70 ms).
-constexpr int kMaxCutDepth = 8, kMaxCuts = 7, kMaxCutsFew = 11, kFewSources = 20;
+// with 11; with 11 for 27 sources per warp 4.93 instead of 4.70 ms). Rechecked with the
+// branch-free step, 5 / 7 / 10 cuts: cube 5.47 / 5.59 / 6.29, clusters 5.89 / 6.02 / 6.25,
+// batch 9.81 / 10.09 / 10.55, slab 48.4 / 48.4 / 48.5: hence 5.
+constexpr int kMaxCutDepth = 8, kMaxCuts = 5, kMaxCutsFew = 11, kFewSources = 20;
 // The default also looks at how many sources the update has, per resident warp of
 // the union kernel (W = 9,728 on 152 SMs at 8 blocks per SM; the sweeps below were
 // taken at 6 blocks, W = 7,296, and the threshold rechecked at 8). Per-update sweeps
@@ -337,6 +343,19 @@ __device__ __forceinline__ void kahan_add(float &sum, float &c, float a)
     sum = t;
 }
 
+// The same where take holds, without a branch: the sum is formed by every lane and kept by
+// the lanes that take it. A walk's step then has no divergent block whose end it waits
+// for (search of the first updates, ms, branch -> select: 2^20 cube 6.30 + 3.25 -> 5.92 +
+// 2.97, 2^22 slab 52.0 + 23.9 -> 48.7 + 22.6, 300,007 neurons at theta 0.2 4.77 + 3.60 ->
+// 4.49 + 3.15, 2^20 clusters 6.64 + 3.61 -> 6.33 + 3.31).
+__device__ __forceinline__ void kahan_take(float &sum, float &c, float a, bool take)
+{
+    float s1 = sum, c1 = c;
+    kahan_add(s1, c1, a);
+    sum = take ? s1 : sum;
+    c = take ? c1 : c;
+}
+
 template <bool kCount>
 __device__ __forceinline__ void union_step(const Node *__restrict__ nodes, int32_t &p,
                                            int32_t &skip, float &cum, float &comp,
@@ -350,10 +369,9 @@ __device__ __forceinline__ void union_step(const Node *__restrict__ nodes, int32
     const bool on = p >= skip && g.w > 0.0f;
     const bool pass = __float_as_uint(d2) + (uint32_t)t.y > thr0;
     if (kCount) own += on ? 1 : 0;
-    if (on && pass) {
-        skip = t.x;
-        if (p != self_node) kahan_add(cum, comp, attraction(g.w, d2, k2, k2sh));
-    }
+    const bool acc = on && pass;
+    if (acc) skip = t.x;
+    kahan_take(cum, comp, attraction(g.w, d2, k2, k2sh), acc && p != self_node);
     // escapes lie past their node in every well-formed tree; the caller checks that each
     // block of steps advances, which keeps the walk finite regardless
     p = __any_sync(0xffffffffu, on && !pass) ? p + 1 : t.x;
@@ -361,28 +379,26 @@ __device__ __forceinline__ void union_step(const Node *__restrict__ nodes, int32
 
 // One step of several union walks in one warp (lane groups gmask; see
 // bh_search_kernel): a group whose walk has ended sits on the sentinel node at
-// root_end, which has no count, and its escape is clamped back to root_end.
+// root_end, which has no count and escapes to itself.
 template <bool kCount>
 __device__ __forceinline__ void group_step(const Node *__restrict__ nodes, int32_t &p,
                                            int32_t &skip, float &cum, float &comp,
-                                           int32_t &own, int32_t &gst, float3 x,
-                                           int32_t self_node, uint32_t thr0, float k2,
-                                           float k2sh, uint32_t gmask, int32_t root_end)
+                                           int32_t &own, float3 x, int32_t self_node,
+                                           uint32_t thr0, float k2, float k2sh,
+                                           uint32_t gmask)
 {
     float4 g;
     int2 t;
-    if (kCount) gst += p < root_end ? 1 : 0;
     load_node(&nodes[p], g, t);
     const float d2 = dist2(x, g);
     const bool on = p >= skip && g.w > 0.0f;
     const bool pass = __float_as_uint(d2) + (uint32_t)t.y > thr0;
     if (kCount) own += on ? 1 : 0;
-    if (on && pass) {
-        skip = t.x;
-        if (p != self_node) kahan_add(cum, comp, attraction(g.w, d2, k2, k2sh));
-    }
+    const bool acc = on && pass;
+    if (acc) skip = t.x;
+    kahan_take(cum, comp, attraction(g.w, d2, k2, k2sh), acc && p != self_node);
     const uint32_t down = __ballot_sync(0xffffffffu, on && !pass) & gmask;
-    p = min(down ? p + 1 : t.x, root_end);
+    p = down ? p + 1 : t.x;
 }
 
 // Draw on the root frontier from a checkpoint: the lane's own walk with pass 1's
@@ -401,12 +417,11 @@ __device__ __forceinline__ int32_t find_root(const Node *__restrict__ nodes, int
         const float d2 = dist2(x, g);
         const bool has = g.w > 0.0f;
         const bool acc = has && (__float_as_uint(d2) + (uint32_t)t.y > thr0);
-        if (acc && p != self_node) {
-            const float a = attraction(g.w, d2, k2, k2sh);
-            kahan_add(cum, comp, a);
-            if (a > 0.0f) pick = p;
-            if (__fsub_rn(cum, comp) > target) return p;
-        }
+        const bool take = acc && p != self_node;
+        const float a = attraction(g.w, d2, k2, k2sh);
+        kahan_take(cum, comp, a, take);
+        pick = take && a > 0.0f ? p : pick;
+        if (take && __fsub_rn(cum, comp) > target) return p;
         p = (has && !acc) ? p + 1 : max(t.x, p + 1);
     }
     return pick;
@@ -590,6 +605,7 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
         int32_t own = 0, nck = 0, task_steps = 0;
         for (int attempt = 0; attempt < 2; ++attempt) {
             int32_t p = root + 1, skip = live ? 0 : 0x7fffffff, steps = 0;
+            int32_t wst = 0; // this walk's own steps (counted with kCount only)
             float cum = 0.0f, comp = 0.0f; // Kahan sum and compensation
             int32_t ckst = 0; // checkpoints stored (bits 0-7) and log2 of the interval in
                               // blocks (bits 8-15): no further live register in the walk
@@ -616,24 +632,23 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
                     checkpoint(max(p, skip));
                     const int32_t p_blk = p;
                     int k = 0;
-                    // four steps per test: nodes root_end .. root_end + 2 are sentinels
-                    // (no count, escape = next node), so steps past the end change nothing
+                    // four steps per test: node root_end is a sentinel (no count, escape =
+                    // itself), so steps past the end change nothing
 #pragma unroll 1
                     for (; k < kCkStride && p < root_end; k += 4) {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                        for (int u = 0; u < 4; ++u) {
+                            if (kCount) wst += p < root_end ? 1 : 0;
                             union_step<kCount>(a.nodes, p, skip, cum, comp, own, x, self_node,
                                                thr0, k2, k2sh);
+                        }
                     }
                     steps += k;
                     if (p <= p_blk) break; // no progress: only a malformed tree
                 }
-                if (p > root_end) steps -= p - root_end; // the sentinels' steps
             } else {
                 // several walks per warp (lane groups gmask) in the same blocks of four
-                // steps per test: a group that has finished parks on the sentinel at
-                // root_end (no count; its escape is clamped back to root_end)
-                int32_t gst = 0; // this group's own steps (counted with kCount only)
+                // steps per test: a group that has finished parks on the sentinel
                 while (__any_sync(0xffffffffu, p < root_end)) {
                     if (p < root_end) checkpoint(max(p, skip));
                     const int32_t p_blk = p;
@@ -641,17 +656,18 @@ __global__ void __launch_bounds__(256, RELEARN_SEARCH_MIN_BLOCKS) bh_search_kern
 #pragma unroll 1
                     for (; k < kCkStride && __any_sync(0xffffffffu, p < root_end); k += 4) {
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            group_step<kCount>(a.nodes, p, skip, cum, comp, own, gst, x,
-                                               self_node, thr0, k2, k2sh, gmask, root_end);
+                        for (int u = 0; u < 4; ++u) {
+                            if (kCount) wst += p < root_end ? 1 : 0;
+                            group_step<kCount>(a.nodes, p, skip, cum, comp, own, x, self_node,
+                                               thr0, k2, k2sh, gmask);
+                        }
                     }
                     steps += k;
                     // no progress: only a malformed tree
                     if (__any_sync(0xffffffffu, p < root_end && p <= p_blk)) break;
                 }
-                steps = gst;
             }
-            if (kCount && lane == seg_first) task_steps += steps; // one count per walk
+            if (kCount && lane == seg_first) task_steps += wst; // one count per walk
             nck = ckst & 0xff;
             S = (double)cum - (double)comp;
             // every term underflowed: redo with the exponents shifted by the nearest d^2
@@ -904,17 +920,14 @@ __device__ __forceinline__ int split_walk(const SearchArgs &a, SplitLists &L, in
             const bool has = g.w > 0.0f;
             const bool acc = has && (__float_as_uint(d2) + (uint32_t)t.y > thr0);
             if (kCount) own += has ? 1 : 0;
-            if (acc && p != self_node) {
-                kahan_add(cum, comp, attraction(g.w, d2, k2, k2sh));
-                dmin2 = fminf(dmin2, d2);
-            }
-            if (has && !acc) { // descend; the part after p's subtree may go to another lane
-                rest = max(t.x, p + 1);
-                split = e - rest >= kSplitMinRest;
-                p = p + 1;
-            } else {
-                p = max(t.x, p + 1);
-            }
+            const bool take = acc && p != self_node;
+            kahan_take(cum, comp, attraction(g.w, d2, k2, k2sh), take);
+            dmin2 = take ? fminf(dmin2, d2) : dmin2;
+            // descend; the part after p's subtree may go to another lane
+            const bool down = has && !acc;
+            rest = max(t.x, p + 1);
+            split = down && e - rest >= kSplitMinRest;
+            p = down ? p + 1 : rest;
             if (p >= e) { // range done
                 L.done(rid, __fsub_rn(cum, comp), rnext);
                 busy = false;
