@@ -276,7 +276,7 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(scan.flags, scan_blocks + 3);
 #undef A
     if (e == cudaSuccess) {
-        for (auto init : {octree_init, search_init, synapses_init})
+        for (auto init : {octree_init, search_init, synapses_init, length_init})
             if (e == cudaSuccess) e = init();
         c->scan.max_blocks = scan_blocks;
         c->scan.status = c->d_status;

@@ -207,6 +207,7 @@ int64_t sort_scratch_words(int64_t blocks);
 cudaError_t octree_init();
 cudaError_t search_init();
 cudaError_t synapses_init();
+cudaError_t length_init();
 
 // octree.cu -----------------------------------------------------------------
 cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, const float *y,

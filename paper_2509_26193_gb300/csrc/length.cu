@@ -31,8 +31,9 @@
 // Measured (GB300, uniform cube, theta 0.3, the forward and backward calls with their
 // small kernels, one-node-per-step union walks -> group walks): 2^18 neurons forward
 // 1.77 -> 1.55 ms, backward 5.75 -> 2.66 ms; 5,003 neurons, forward + backward
-// 5.5 -> 0.24 ms. Bound by instruction issue (70 to 73 % active at 2^18: per entry and
+// 5.5 -> 0.18 ms. Bound by instruction issue (70 to 73 % active at 2^18: per entry and
 // group about 16 instructions of forward sums, 40 of backward ones, and 16 of walking).
+#include "cluster.cuh"
 #include "internal.h"
 
 namespace rl {
@@ -868,62 +869,115 @@ __device__ __forceinline__ int32_t sibling_rank(const Node *__restrict__ nodes, 
 }
 
 // Child counts: a node's last child (same escape) knows its own rank. Leaves have none.
-__global__ void family_count_kernel(const Node *__restrict__ nodes,
-                                    const int32_t *__restrict__ parent,
-                                    const int64_t *d_num_nodes, int32_t *__restrict__ count)
+__device__ __forceinline__ void family_count(const Node *__restrict__ nodes,
+                                             const int32_t *__restrict__ parent, int32_t v,
+                                             int32_t *count)
 {
-    const int64_t m = *d_num_nodes;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < m;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const NodeTopo t = nodes[v].t;
-        if (node_is_leaf(t.shift)) count[v] = 0;
-        const int32_t u = parent[v];
-        if (u >= 0 && nodes[u].t.escape == t.escape)
-            count[u] = sibling_rank(nodes, u, (int32_t)v) + 1;
+    const NodeTopo t = nodes[v].t;
+    if (node_is_leaf(t.shift)) count[v] = 0;
+    const int32_t u = parent[v];
+    if (u >= 0 && nodes[u].t.escape == t.escape) count[u] = sibling_rank(nodes, u, v) + 1;
+}
+
+__device__ __forceinline__ void family_emit(const Node *__restrict__ nodes,
+                                            const int32_t *__restrict__ parent, int32_t v,
+                                            const int32_t *k0, FamNode *fam)
+{
+    const Node nd = nodes[v];
+    const int32_t u = parent[v];
+    const bool last = u < 0 || nodes[u].t.escape == nd.t.escape;
+    FamNode f;
+    f.cx = nd.g.cx;
+    f.cy = nd.g.cy;
+    f.cz = nd.g.cz;
+    f.cnt = nd.g.cnt;
+    f.pre = v;
+    f.up = u;
+    f.kids = node_is_leaf(nd.t.shift) ? 0u : (uint32_t)(1 + k0[v]);
+    f.shift = nd.t.shift | (last ? kLastSibling : 0u);
+    fam[u < 0 ? 0 : 1 + k0[u] + sibling_rank(nodes, u, v)] = f;
+}
+
+// What a forward pass sets up: the active sources (vac_ax > 0) in Morton order, the tree
+// in family order with the geometry the bottom-up update just formed, its sums and its
+// work counter zeroed: the steps before and after the two prefix sums (over flag and k0),
+// or, for networks of at most kSmallLen neurons, all of it as one cluster kernel. Whole
+// forward call on the device, us, with a launch for each step -> with two kernels and two
+// prefix sums -> with the cluster kernel: 1,000 neurons 71 -> 62 -> 52, 5,003 105 -> 97 ->
+// 86, 16,000 151 -> 142 -> 138, 24,000 206 -> 200 -> 199, 40,000 320 -> 311 -> 317.
+struct PrepArgs {
+    const int32_t *vac_ax, *perm;
+    int64_t n;
+    int32_t *flag, *off, *act_src;
+    int64_t *active;
+    const Node *nodes;
+    const int32_t *parent;
+    const int64_t *d_num_nodes;
+    int32_t *k0;
+    FamNode *fam;
+    double *lsum;
+    int32_t *work;
+};
+constexpr int64_t kSmallLen = 16384;
+
+#define GRID_STRIDE(i, n)                                                                         \
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n);                     \
+         i += (int64_t)gridDim.x * blockDim.x)
+#define CLUSTER_STRIDE(i, n)                                                                      \
+    for (int64_t i = cluster_form::first(); i < (n); i += cluster_form::kStride)
+
+__device__ __forceinline__ int32_t active_flag(const PrepArgs &a, int64_t s)
+{
+    return a.vac_ax[a.perm[s]] > 0 ? 1 : 0;
+}
+
+__device__ __forceinline__ void clear_sums(const PrepArgs &a)
+{
+    for (int k = 0; k < 4; ++k) a.lsum[k] = 0.0;
+    *a.work = 0;
+}
+
+__global__ void len_count_kernel(PrepArgs a)
+{
+    const int64_t m = *a.d_num_nodes;
+    if (blockIdx.x == 0 && threadIdx.x == 0) clear_sums(a);
+    GRID_STRIDE(s, a.n + 1) a.flag[s] = s < a.n ? active_flag(a, s) : 0;
+    GRID_STRIDE(v, m) family_count(a.nodes, a.parent, (int32_t)v, a.k0);
+}
+
+__global__ void len_emit_kernel(PrepArgs a)
+{
+    const int64_t m = *a.d_num_nodes;
+    GRID_STRIDE(s, a.n)
+    {
+        if (a.flag[s]) a.act_src[a.off[s]] = (int32_t)s;
     }
+    GRID_STRIDE(v, m) family_emit(a.nodes, a.parent, (int32_t)v, a.k0, a.fam);
 }
 
-__global__ void family_emit_kernel(const Node *__restrict__ nodes,
-                                   const int32_t *__restrict__ parent,
-                                   const int64_t *d_num_nodes, const int32_t *__restrict__ k0,
-                                   FamNode *__restrict__ fam)
+__global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
+    __launch_bounds__(cluster_form::kThreads) len_prepare_small_kernel(PrepArgs a)
 {
-    const int64_t m = *d_num_nodes;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < m;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const Node nd = nodes[v];
-        const int32_t u = parent[v];
-        const bool last = u < 0 || nodes[u].t.escape == nd.t.escape;
-        FamNode f;
-        f.cx = nd.g.cx;
-        f.cy = nd.g.cy;
-        f.cz = nd.g.cz;
-        f.cnt = nd.g.cnt;
-        f.pre = (int32_t)v;
-        f.up = u;
-        f.kids = node_is_leaf(nd.t.shift) ? 0u : (uint32_t)(1 + k0[v]);
-        f.shift = nd.t.shift | (last ? kLastSibling : 0u);
-        fam[u < 0 ? 0 : 1 + k0[u] + sibling_rank(nodes, u, (int32_t)v)] = f;
+    namespace cf = cluster_form;
+    const int64_t m = *a.d_num_nodes;
+    CLUSTER_STRIDE(v, m) family_count(a.nodes, a.parent, (int32_t)v, a.k0);
+    const cf::I32 total = cf::scan<cf::I32>(
+        a.n, [&](int64_t s) { return cf::I32{a.flag[s] = active_flag(a, s)}; },
+        [&](int64_t s) { return cf::I32{a.flag[s]}; },
+        [&](int64_t s, cf::I32 prefix, cf::I32 on, cf::I32) {
+            if (on.v) a.act_src[prefix.v] = (int32_t)s;
+        });
+    if (cf::first() == 0) {
+        clear_sums(a);
+        *a.active = total.v;
     }
-}
-
-// Active sources (vac_ax > 0) in Morton order.
-__global__ void len_flags_kernel(const int32_t *__restrict__ vac_ax,
-                                 const int32_t *__restrict__ perm, int64_t n,
-                                 int32_t *__restrict__ flag)
-{
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= n;
-         s += (int64_t)gridDim.x * blockDim.x)
-        flag[s] = s < n && vac_ax[perm[s]] > 0 ? 1 : 0;
-}
-
-__global__ void len_fill_kernel(const int32_t *__restrict__ flag,
-                                const int32_t *__restrict__ off, int64_t n,
-                                int32_t *__restrict__ act_src)
-{
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x)
-        if (flag[s]) act_src[off[s]] = (int32_t)s;
+    cf::sync(); // the child counts and the scan's shared words
+    cf::scan<cf::I32>(
+        m, [&](int64_t v) { return cf::I32{a.k0[v]}; },
+        [&](int64_t v) { return cf::I32{a.k0[v]}; },
+        [&](int64_t v, cf::I32 prefix, cf::I32, cf::I32) { a.k0[v] = prefix.v; });
+    cf::sync();
+    CLUSTER_STRIDE(v, m) family_emit(a.nodes, a.parent, (int32_t)v, a.k0, a.fam);
 }
 
 // mean = sum m l / M (NaN when M = 0); ell[id] = l (NaN for excluded neurons).
@@ -945,41 +999,72 @@ __global__ void len_finish_kernel(const float4 *__restrict__ state,
     }
 }
 
-__global__ void zero_nodes_kernel(double4 *G, const int64_t *d_num_nodes)
+// What a backward pass adds into, zeroed in one launch.
+__global__ void len_zero_kernel(double4 *G, const int64_t *d_num_nodes, int64_t n, float *gx,
+                                float *gy, float *gz, double *gsigma, int32_t *work)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *work = 0;
+        if (gsigma) *gsigma = 0.0;
+    }
     const int64_t m = *d_num_nodes;
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m;
-         k += (int64_t)gridDim.x * blockDim.x)
-        G[k] = make_double4(0.0, 0.0, 0.0, 0.0);
+    GRID_STRIDE(k, m) G[k] = make_double4(0.0, 0.0, 0.0, 0.0);
+    GRID_STRIDE(i, n) gx[i] = gy[i] = gz[i] = 0.0f;
 }
 
-// Neuron j (Morton position s) gets w_j * sum over its cells k of G_k / N_k.
-__global__ void len_scatter_kernel(const Node *__restrict__ nodes,
-                                   const int32_t *__restrict__ parent,
-                                   const int32_t *__restrict__ leaf_of,
-                                   const int32_t *__restrict__ perm,
-                                   const int32_t *__restrict__ vac_de, const double *__restrict__ G,
-                                   int64_t n, float *gx, float *gy, float *gz)
+// Neuron j (Morton position s) gets w_j * sum over its cells k of G_k / N_k: first G / N
+// per node (a node without vacant elements is no candidate and has G = 0), then every
+// neuron's sum up its parent chain. One FP64 division per node instead of one per neuron
+// and level. Whole backward call on the device with this and the zeroing in one launch:
+// 1,000 neurons 59 -> 49 us, 5,003 106 -> 96, 40,000 460 -> 448, 2^18 2,773 -> 2,761. (As
+// one cluster kernel: 50, 99, 481.)
+struct ScatterArgs {
+    const Node *nodes;
+    const int32_t *parent, *leaf_of, *perm, *vac_de;
+    const int64_t *d_num_nodes;
+    double *G;
+    int64_t n;
+    float *gx, *gy, *gz;
+};
+
+__device__ __forceinline__ void scale_node(const ScatterArgs &a, int64_t u)
 {
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t i = perm[s];
-        const int32_t w = vac_de[i];
-        if (w <= 0) continue;
-        double hx = 0.0, hy = 0.0, hz = 0.0;
-        for (int32_t u = leaf_of[s]; u >= 0; u = parent[u]) {
-            const int32_t cnt = nodes[u].t.icount;
-            if (cnt <= 0) continue;
-            const double inv = 1.0 / (double)cnt;
-            hx += G[4 * (int64_t)u + 0] * inv;
-            hy += G[4 * (int64_t)u + 1] * inv;
-            hz += G[4 * (int64_t)u + 2] * inv;
-        }
-        // direct term (FP32) + cell terms (FP64), rounded once
-        gx[i] = (float)((double)gx[i] + w * hx);
-        gy[i] = (float)((double)gy[i] + w * hy);
-        gz[i] = (float)((double)gz[i] + w * hz);
+    const int32_t cnt = a.nodes[u].t.icount;
+    if (cnt <= 0) return;
+    const double inv = 1.0 / (double)cnt;
+    double *g = a.G + 4 * u;
+    g[0] *= inv;
+    g[1] *= inv;
+    g[2] *= inv;
+}
+
+__device__ __forceinline__ void gather_chain(const ScatterArgs &a, int64_t s)
+{
+    const int32_t i = a.perm[s];
+    const int32_t w = a.vac_de[i];
+    if (w <= 0) return;
+    double hx = 0.0, hy = 0.0, hz = 0.0;
+    for (int32_t u = a.leaf_of[s]; u >= 0; u = a.parent[u]) {
+        const double *g = a.G + 4 * (int64_t)u;
+        hx += g[0];
+        hy += g[1];
+        hz += g[2];
     }
+    // direct term (FP32) + cell terms (FP64), rounded once
+    a.gx[i] = (float)((double)a.gx[i] + w * hx);
+    a.gy[i] = (float)((double)a.gy[i] + w * hy);
+    a.gz[i] = (float)((double)a.gz[i] + w * hz);
+}
+
+__global__ void len_scale_kernel(ScatterArgs a)
+{
+    const int64_t m = *a.d_num_nodes;
+    GRID_STRIDE(u, m) scale_node(a, u);
+}
+
+__global__ void len_scatter_kernel(ScatterArgs a)
+{
+    GRID_STRIDE(s, a.n) gather_chain(a, s);
 }
 
 LenArgs make_args(relearn_ctx *c, const int32_t *vac_ax)
@@ -1004,8 +1089,6 @@ LenArgs make_args(relearn_ctx *c, const int32_t *vac_ax)
 template <bool kBack>
 cudaError_t launch_length(relearn_ctx *c, const LenArgs &a, cudaStream_t st)
 {
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(c->d_i32 + I32_WORK, 0, sizeof(int32_t), st))) return e;
     length_kernel<kBack>
         <<<c->num_sms * RELEARN_LEN_MIN_BLOCKS, 32 * kGroupWarps, 0, st>>>(a);
     note_launch();
@@ -1019,33 +1102,39 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
 {
     cudaError_t e;
     const int64_t n = c->n;
-    int32_t *flag = c->d_cnt;
-    len_flags_kernel<<<grid_for(n + 1, 256, c->num_sms), 256, 0, st>>>(vac_ax, c->d_perm, n,
-                                                                        flag);
-    note_launch();
-    if ((e = scan_exclusive(flag, c->d_act_off, n + 1, nullptr, c->d_i64 + I64_ACTIVE, c->scan,
-                            st)))
-        return e;
-    len_fill_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(flag, c->d_act_off, n,
-                                                                   c->d_act_src);
-    note_launch();
-    // the tree in family order, with the geometry the bottom-up update just formed (its
-    // prefix scratch is free again)
-    int32_t *k0 = reinterpret_cast<int32_t *>(c->d_acc);
-    const unsigned gm = grid_for(2 * n + 1, 256, c->num_sms);
-    family_count_kernel<<<gm, 256, 0, st>>>(c->d_nodes, c->d_parent, c->d_i64 + I64_NODES, k0);
-    note_launch();
-    // the node count as int32 (its low word)
-    if ((e = scan_exclusive(k0, k0, 2 * n + 1,
-                            reinterpret_cast<const int32_t *>(c->d_i64 + I64_NODES), nullptr,
-                            c->scan, st)))
-        return e;
-    family_emit_kernel<<<gm, 256, 0, st>>>(c->d_nodes, c->d_parent, c->d_i64 + I64_NODES, k0,
-                                           c->d_fam);
-    note_launch();
-    if ((e = cudaMemsetAsync(c->d_lsum, 0, 4 * sizeof(double), st))) return e;
+    PrepArgs p;
+    p.vac_ax = vac_ax;
+    p.perm = c->d_perm;
+    p.n = n;
+    p.flag = c->d_cnt;
+    p.off = c->d_act_off;
+    p.act_src = c->d_act_src;
+    p.active = c->d_i64 + I64_ACTIVE;
+    p.nodes = c->d_nodes;
+    p.parent = c->d_parent;
+    p.d_num_nodes = c->d_i64 + I64_NODES;
+    p.k0 = reinterpret_cast<int32_t *>(c->d_acc); // the bottom-up update's scratch is free
+    p.fam = c->d_fam;
+    p.lsum = c->d_lsum;
+    p.work = c->d_i32 + I32_WORK;
+    if (n <= kSmallLen) {
+        len_prepare_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(p);
+        note_launch();
+    } else {
+        const unsigned gm = grid_for(2 * n + 1, 256, c->num_sms);
+        len_count_kernel<<<gm, 256, 0, st>>>(p);
+        note_launch();
+        if ((e = scan_exclusive(p.flag, p.off, n + 1, nullptr, p.active, c->scan, st))) return e;
+        // the node count as int32 (its low word)
+        if ((e = scan_exclusive(p.k0, p.k0, 2 * n + 1,
+                                reinterpret_cast<const int32_t *>(p.d_num_nodes), nullptr,
+                                c->scan, st)))
+            return e;
+        len_emit_kernel<<<gm, 256, 0, st>>>(p);
+        note_launch();
+    }
     if ((e = launch_length<false>(c, make_args(c, vac_ax), st))) return e;
-    len_finish_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(c->d_lstate, flag,
+    len_finish_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(c->d_lstate, p.flag,
                                                                      c->d_perm, n, c->d_lsum,
                                                                      ell, mean);
     note_launch();
@@ -1060,12 +1149,10 @@ cudaError_t length_backward(relearn_ctx *c, const int32_t *vac_ax, const int32_t
     const int64_t n = c->n;
     // d_acc is free between bottom-up updates (32 bytes per node: x, y, z in FP64)
     double *G = c->d_acc;
-    zero_nodes_kernel<<<grid_for(c->max_nodes, 256, c->num_sms), 256, 0, st>>>(
-        reinterpret_cast<double4 *>(G), c->d_i64 + I64_NODES);
+    len_zero_kernel<<<grid_for(2 * n, 256, c->num_sms), 256, 0, st>>>(
+        reinterpret_cast<double4 *>(G), c->d_i64 + I64_NODES, n, gx, gy, gz, gsigma,
+        c->d_i32 + I32_WORK);
     note_launch();
-    for (float *g : {gx, gy, gz})
-        if ((e = cudaMemsetAsync(g, 0, n * sizeof(float), st))) return e;
-    if (gsigma && (e = cudaMemsetAsync(gsigma, 0, sizeof(double), st))) return e;
     LenArgs a = make_args(c, vac_ax);
     a.G = G;
     a.gx = gx;
@@ -1074,10 +1161,18 @@ cudaError_t length_backward(relearn_ctx *c, const int32_t *vac_ax, const int32_t
     a.gout = grad_mean;
     a.gsigma = gsigma;
     if ((e = launch_length<true>(c, a, st))) return e;
-    len_scatter_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(
-        c->d_nodes, c->d_parent, c->d_leaf, c->d_perm, vac_de, G, n, gx, gy, gz);
+    const ScatterArgs s{c->d_nodes, c->d_parent, c->d_leaf, c->d_perm, vac_de,
+                        c->d_i64 + I64_NODES, G, n, gx, gy, gz};
+    len_scale_kernel<<<grid_for(2 * n, 256, c->num_sms), 256, 0, st>>>(s);
+    note_launch();
+    len_scatter_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(s);
     note_launch();
     return cudaGetLastError();
+}
+
+cudaError_t length_init()
+{
+    return cluster_form::allow(len_prepare_small_kernel);
 }
 
 } // namespace rl
