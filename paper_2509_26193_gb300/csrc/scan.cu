@@ -19,6 +19,14 @@ constexpr int kThreads = 256;
 constexpr int kItems = 16;
 constexpr int kTile = kThreads * kItems;
 
+// Place of the tile's element e in shared memory: a thread's 16 neighbours start at 16 t,
+// which without the shift puts a warp's reads on two banks. With it, the tile states
+// cleared up to the last one used and no second ticket where every tile has a block, an
+// update with deletion of 50,021 clustered neurons (16 scans) takes 2.17 instead of
+// 2.20 ms, ten updates of 2^20 (24 scans) 15.31 instead of 15.42 ms. (Sum and state of a
+// tile in one 64-bit word, or fewer blocks per SM: the same.)
+__device__ __forceinline__ int at(int e) { return e + (e >> 5); }
+
 __device__ __forceinline__ int64_t bounded_count(int64_t max_n, const int32_t *d_count)
 {
     if (!d_count) return max_n;
@@ -72,16 +80,17 @@ __device__ __forceinline__ void scan_tile(const int32_t *in, int32_t *out, int64
                                           int32_t *tile, int64_t &s_prefix)
 {
     const int64_t base = t * kTile;
+#pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const int64_t i = base + (int64_t)k * kThreads + threadIdx.x;
-        tile[k * kThreads + threadIdx.x] = i < n ? in[i] : 0;
+        tile[at(k * kThreads + threadIdx.x)] = i < n ? in[i] : 0;
     }
     __syncthreads();
     int32_t v[kItems];
     int64_t s = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
-        v[k] = tile[threadIdx.x * kItems + k];
+        v[k] = tile[at(threadIdx.x * kItems + k)];
         s += v[k];
     }
     int64_t tot;
@@ -185,13 +194,14 @@ __device__ __forceinline__ void scan_tile(const int32_t *in, int32_t *out, int64
     int64_t run = s_prefix + incl - s;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
-        tile[threadIdx.x * kItems + k] = (int32_t)run;
+        tile[at(threadIdx.x * kItems + k)] = (int32_t)run;
         run += v[k];
     }
     __syncthreads();
+#pragma unroll
     for (int k = 0; k < kItems; ++k) {
         const int64_t i = base + (int64_t)k * kThreads + threadIdx.x;
-        if (i < n) out[i] = tile[k * kThreads + threadIdx.x];
+        if (i < n) out[i] = tile[at(k * kThreads + threadIdx.x)];
     }
 }
 
@@ -199,10 +209,9 @@ __global__ void __launch_bounds__(kThreads)
     scan_kernel(const int32_t *in, int32_t *out, int64_t max_n, const int32_t *d_count,
                 int32_t *flags, int64_t *agg, int64_t *inc, int64_t *d_total, int32_t *status)
 {
-    __shared__ int32_t tile[kTile];
+    __shared__ int32_t tile[kTile + kTile / 32];
     __shared__ int64_t s_prefix;
     __shared__ int32_t s_t, s_last;
-    const int64_t max_tiles = max_n > 0 ? (max_n + kTile - 1) / kTile : 1;
     if (threadIdx.x == 0) s_t = atomicAdd(&flags[0], 1);
     __syncthreads();
     const int64_t n = bounded_count(max_n, d_count);
@@ -213,6 +222,7 @@ __global__ void __launch_bounds__(kThreads)
     // only waits for smaller tickets, held by blocks already running)
     for (int64_t t = s_t; t <= last_tile;) {
         scan_tile(in, out, n, t, last_tile, flags, agg, inc, d_total, status, tile, s_prefix);
+        if (last_tile < gridDim.x) break;
         __syncthreads();
         if (threadIdx.x == 0) s_t = atomicAdd(&flags[0], 1);
         __syncthreads();
@@ -227,7 +237,7 @@ __global__ void __launch_bounds__(kThreads)
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (int64_t j = threadIdx.x; j < max_tiles; j += blockDim.x) flags[3 + j] = 0;
+        for (int64_t j = threadIdx.x; j <= last_tile; j += blockDim.x) flags[3 + j] = 0;
         if (threadIdx.x == 0) {
             flags[0] = 0;
             flags[1] = 0;
