@@ -442,21 +442,25 @@ __device__ __forceinline__ Four four_of(const int32_t *__restrict__ a, int64_t q
     return f;
 }
 
+__device__ __forceinline__ void four_spikes(int64_t q, int64_t m, const int32_t *src,
+                                            const int32_t *tgt, const int8_t *sign,
+                                            const uint8_t *spiked, int32_t *input)
+{
+    const Four s = four_of(src, q, m, -1);
+    uint8_t on[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) on[k] = s.v[k] >= 0 ? spiked[s.v[k]] : 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (on[k]) atomicAdd(&input[tgt[4 * q + k]], (int32_t)sign[4 * q + k]);
+}
+
 __global__ void spikes_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
                               const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
                               const uint8_t *__restrict__ spiked, int32_t *__restrict__ input)
 {
     const int64_t m = *d_nsyn;
-    GRID_STRIDE(q, (m + 3) / 4)
-    {
-        const Four s = four_of(src, q, m, -1);
-        uint8_t on[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) on[k] = s.v[k] >= 0 ? spiked[s.v[k]] : 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (on[k]) atomicAdd(&input[tgt[4 * q + k]], (int32_t)sign[4 * q + k]);
-    }
+    GRID_STRIDE(q, (m + 3) / 4) four_spikes(q, m, src, tgt, sign, spiked, input);
 }
 
 // Firing-rate delivery (Sec. IV-B): the receiver t decides once per step and per
@@ -473,6 +477,21 @@ __device__ __forceinline__ bool rate_fires(int32_t s, int32_t t, float rate, uin
     return rate > 0.0f && w < __float2uint_ru(__fmul_rn(rate, 4294967296.0f)); // NaN: never
 }
 
+__device__ __forceinline__ void four_rates(int64_t q, int64_t m, const int32_t *src,
+                                           const int32_t *tgt, const int8_t *sign,
+                                           const float *rate, uint64_t seed, uint32_t step,
+                                           int32_t *input)
+{
+    const Four s = four_of(src, q, m, -1), t = four_of(tgt, q, m, 0);
+    float r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] = s.v[k] >= 0 ? rate[s.v[k]] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (rate_fires(s.v[k], t.v[k], r[k], seed, step))
+            atomicAdd(&input[t.v[k]], (int32_t)sign[4 * q + k]);
+}
+
 // As spikes_kernel (1.8 million synapses 19.7 -> 14.4 us a call, 3.4 million 31.0 -> 18.6;
 // one, two or four synapses per thread are the same here: the generator bounds it).
 __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
@@ -481,17 +500,7 @@ __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ 
                              int32_t *__restrict__ input)
 {
     const int64_t m = *d_nsyn;
-    GRID_STRIDE(q, (m + 3) / 4)
-    {
-        const Four s = four_of(src, q, m, -1), t = four_of(tgt, q, m, 0);
-        float r[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) r[k] = s.v[k] >= 0 ? rate[s.v[k]] : 0.0f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (rate_fires(s.v[k], t.v[k], r[k], seed, step))
-                atomicAdd(&input[t.v[k]], (int32_t)sign[4 * q + k]);
-    }
+    GRID_STRIDE(q, (m + 3) / 4) four_rates(q, m, src, tgt, sign, rate, seed, step, input);
 }
 
 // ---------------------------------------------------------------- small networks
@@ -710,7 +719,10 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     }
 }
 
-// input = 0, then as spikes_kernel (spiked given) or rates_kernel.
+// input = 0, then as spikes_kernel (spiked given) or rates_kernel: one launch instead of a
+// memset and a kernel (a spike and a rate delivery called in turn, 5,000 to 40,000 neurons:
+// 20.6 -> 16.6 us; replayed from a graph, which has no launch gaps to save, 8.3 to 10.3
+// before, 10.3 to 12.4 now).
 __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     __launch_bounds__(cluster_form::kThreads)
     deliver_small_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
@@ -722,11 +734,12 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     const int64_t m = *d_nsyn;
     CLUSTER_STRIDE(i, n) input[i] = 0;
     cf::sync();
-    CLUSTER_STRIDE(k, m)
+    CLUSTER_STRIDE(q, (m + 3) / 4)
     {
-        const int32_t s = src[k];
-        const bool fires = spiked ? spiked[s] != 0 : rate_fires(s, tgt[k], rate[s], seed, step);
-        if (fires) atomicAdd(&input[tgt[k]], (int32_t)sign[k]);
+        if (spiked)
+            four_spikes(q, m, src, tgt, sign, spiked, input);
+        else
+            four_rates(q, m, src, tgt, sign, rate, seed, step, input);
     }
 }
 
