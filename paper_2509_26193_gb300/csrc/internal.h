@@ -185,7 +185,6 @@ cudaError_t scan_exclusive(const int32_t *in, int32_t *out, int64_t max_n, const
                            int64_t *d_total, ScanScratch &s, cudaStream_t st);
 int64_t scan_blocks_needed(int64_t max_n);
 int64_t scan_grid_cap(int num_sms);
-cudaError_t fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t st);
 
 // sort.cu -------------------------------------------------------------------
 // Stable LSD radix sort of (key, val) on bits [0, end_bit). Returns the buffer

@@ -245,13 +245,6 @@ __global__ void __launch_bounds__(kThreads)
         }
     }
 }
-
-__global__ void fill_kernel(int32_t *p, int32_t v, int64_t n)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = v;
-}
 } // namespace
 
 int64_t scan_blocks_needed(int64_t max_n) { return (max_n + kTile - 1) / kTile; }
@@ -278,16 +271,6 @@ cudaError_t scan_exclusive(const int32_t *in, int32_t *out, int64_t max_n, const
     scan_kernel<<<(unsigned)grid, kThreads, 0, st>>>(in, out, max_n, d_count, s.flags,
                                                      s.block_sums, s.block_sums + nb, d_total,
                                                      s.status);
-    note_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t st)
-{
-    if (n <= 0) return cudaSuccess;
-    int64_t blocks = (n + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    fill_kernel<<<(unsigned)blocks, 256, 0, st>>>(p, v, n);
     note_launch();
     return cudaGetLastError();
 }

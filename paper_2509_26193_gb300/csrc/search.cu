@@ -57,7 +57,7 @@ constexpr float kTiny = 8.673617e-19f; // 2^-60
 // the boundaries of cells of some depth, and each piece walks one union: finer pieces
 // make shorter walks, but every piece reads its own node at each step. The depth is
 // chosen per warp: the deepest one, up to kMaxCutDepth, that leaves at most kMaxCuts cuts
-// (four sources a piece; one depth for every warp suits one density: depth 6 is the best
+// (five to six sources a piece; one depth for every warp suits one density: depth 6 is the best
 // in the 2^20 clusters and the 2^22 slab, depth 5 in a 2^20 cube). Search of the first
 // updates, ms, one depth 6 (a batch: 2) -> at most 2 / 4 / 7 / 10 / 15 cuts: 2^20 cube
 // 6.72 + 4.00 -> 6.35 + 3.51 / 6.34 + 3.28 / 6.33 + 3.30 / 6.67 + 3.31 / 6.74 + 3.60; 2^22
@@ -65,7 +65,7 @@ constexpr float kTiny = 8.673617e-19f; // 2^-60
 // 300,007 clustered neurons at theta 0.2 4.92 + 3.67 -> 4.68 + 3.64 with 7; 2^20 clusters
 // 6.51 + 3.65 -> 6.56 + 3.57 / 6.63 + 3.64 / 6.64 + 3.59 / 6.75 + 3.62 / 7.40 + 3.81;
 // batch of 64 networks 14.5 -> 11.2 with 7 (most of it the blocks of four steps, which a
-// batch takes too since every network has its own sentinels). Updates with at most
+// batch takes too since every network has its own sentinel). Updates with at most
 // kFewSources sources per resident warp wait on their longest walks rather than on the
 // reads of many pieces: kMaxCutsFew (third update of the cube 2.50 -> 2.06 with 7, 1.77
 // with 11; with 11 for 27 sources per warp 4.93 instead of 4.70 ms). Rechecked with the
