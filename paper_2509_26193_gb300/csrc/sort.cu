@@ -19,6 +19,7 @@
 // threads, 4 keys each: 300,000 / 700,001 / 2^20 positions 54 / 76 / 98 us; 8 keys 60 /
 // 80 / 93; 256 threads of 8 keys 59 / 79 / 102, of 16 keys 75 / 108 / 125.
 #include "internal.h"
+#include "tile_state.h"
 
 namespace rl {
 
@@ -36,9 +37,6 @@ constexpr int kMaxPasses = 8;
 constexpr int kItems = RELEARN_SORT_ITEMS;   // keys per thread
 constexpr int kTile = kThreads * kItems;      // keys per block
 constexpr int kSortSpin = 1 << 18;
-
-// A tile's state for one digit: its count, or the inclusive prefix of the counts up to it.
-constexpr uint32_t kStateAgg = 1u << 30, kStateInc = 2u << 30, kStateVal = (1u << 30) - 1;
 
 __device__ __forceinline__ int64_t bounded_count(int64_t max_n, const int32_t *d_count)
 {
@@ -137,7 +135,7 @@ __global__ void __launch_bounds__(kThreads)
                 wcnt[w][d] = cnt;
                 cnt += c;
             }
-            st[tile * kRadix + d] = (tile == 0 ? kStateInc : kStateAgg) | cnt;
+            st[tile * kRadix + d] = tile == 0 ? state_of_prefix(cnt) : state_of_count(cnt);
             total = hist[d];
         }
         // where digit d starts among all keys, and in the tile
@@ -172,24 +170,24 @@ __global__ void __launch_bounds__(kThreads)
                 uint32_t f[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    f[q] = t - q >= 0 ? (uint32_t)st[(t - q) * kRadix + d] : (uint32_t)kStateInc;
+                    f[q] = t - q >= 0 ? (uint32_t)st[(t - q) * kRadix + d] : state_of_prefix(0u);
                 bool done = false;
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    if (done || (f[q] & ~kStateVal) == 0u) break; // not published: read again
-                    prefix += f[q] & kStateVal;
-                    done = (f[q] & kStateInc) != 0u;
+                    if (done || !state_published(f[q])) break; // read again
+                    prefix += state_value(f[q]);
+                    done = state_is_prefix(f[q]);
                     --t;
                 }
                 if (done) break;
-                if ((f[0] & ~kStateVal) == 0u &&
+                if (!state_published(f[0]) &&
                     (++spin >= kSortSpin || *(volatile uint32_t *)abort_ != 0u)) {
                     if (status) set_status(status, RELEARN_ERR_TIMEOUT);
                     *(volatile uint32_t *)abort_ = 1u;
                     break;
                 }
             }
-            if (tile > 0) st[tile * kRadix + d] = kStateInc | ((prefix + cnt) & kStateVal);
+            if (tile > 0) st[tile * kRadix + d] = state_of_prefix(prefix + cnt);
             s_base[d] = start + prefix - loc;
         }
     }
