@@ -87,6 +87,10 @@ __global__ void __launch_bounds__(kThreads)
     for (int i = threadIdx.x; i < kWarps * kRadix; i += kThreads) (&wcnt[0][0])[i] = 0;
     __syncthreads();
     const int64_t tile = s_tile;
+    // Sorts that share scratch and overlap (relearn_morton_order_noalloc states that such
+    // calls race) draw from one ticket counter: their results are void, but no tile past
+    // this grid's has a state to write.
+    if (tile >= gridDim.x) return;
     if (threadIdx.x < kRadix) next_state[tile * kRadix + threadIdx.x] = 0;
     const int64_t tile0 = tile * kTile;
     if (tile0 >= n) return;
