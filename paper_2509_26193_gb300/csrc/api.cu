@@ -293,7 +293,6 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_off, (NB + 1) * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->off_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMemset(c->d_box, 0, sizeof(uint32_t));
     if (e == cudaSuccess)
         e = cudaMemset(c->scan.flags, 0, (c->scan.max_blocks + 3) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_i64, 0, 16 * sizeof(int64_t));

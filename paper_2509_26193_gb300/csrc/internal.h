@@ -78,7 +78,7 @@ struct relearn_ctx {
     int64_t *h_off = nullptr;     // [max_nets + 1] pinned staging of the offsets
     cudaEvent_t off_ev = nullptr; // the last copy out of h_off
     uint32_t *d_ord = nullptr;    // [6 * max_nets] bounding boxes (ordered-int min, max)
-    uint32_t *d_box = nullptr;    // [2048] one network: a count and the blocks' boxes
+    uint32_t *d_box = nullptr;    // [2048] one network: the blocks' boxes
     int32_t *d_root = nullptr;    // [max_nets] root node of each network
     int32_t *d_net = nullptr;     // [n] network of each Morton position (max_nets > 1)
     uint64_t *d_nkey = nullptr, *d_nkey_alt = nullptr; // [n] (network, code) sort keys
@@ -196,6 +196,7 @@ cudaError_t radix_sort_u32(uint32_t *keys, uint32_t *keys_alt, int32_t *vals, in
                            cudaStream_t st, int *which, bool counted = false);
 cudaError_t sort_clear_u32(int64_t n, SortScratch &s, cudaStream_t st);
 uint32_t *sort_counts(SortScratch &s);
+uint32_t *sort_zero_word(SortScratch &s); // one more word that sort_clear_u32 zeroes
 cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int32_t *vals, int32_t *vals_alt,
                            int64_t max_n, const int32_t *d_count, int end_bit, SortScratch &s,
                            cudaStream_t st, int *which);

@@ -158,8 +158,8 @@ __global__ void geom_kernel(const uint32_t *d_ord_all, Box box, Geom *g_all, int
 // One network, one launch: every thread folds its elements into a running min / max, the
 // block reduces them and stores its six words, and the last block to finish reduces the
 // blocks' words and forms the geometry (700,001 positions: 13.2 us in three kernels,
-// 10.0 here). part: [1 + 6 * grid], the first word a count that is zero between calls;
-// off_one: the offsets {0, n}, or NULL.
+// 10.0 here). part: [6 * grid]; done: the blocks that have stored theirs, zeroed before
+// (with the sort's counts); off_one: the offsets {0, n}, or NULL.
 constexpr int kBoxBlocks = 304;
 __device__ __forceinline__ void box_fold(uint32_t v[6], uint32_t (*s_red)[6])
 {
@@ -186,8 +186,8 @@ __device__ __forceinline__ void box_fold(uint32_t v[6], uint32_t (*s_red)[6])
 __global__ void __launch_bounds__(256) box_geom_kernel(const float *__restrict__ x,
                                                        const float *__restrict__ y,
                                                        const float *__restrict__ z, int64_t n,
-                                                       Box box, uint32_t *part, Geom *g,
-                                                       int64_t *off_one)
+                                                       Box box, uint32_t *part, uint32_t *done,
+                                                       Geom *g, int64_t *off_one)
 {
     __shared__ uint32_t s_red[8][6];
     __shared__ bool s_last;
@@ -204,17 +204,17 @@ __global__ void __launch_bounds__(256) box_geom_kernel(const float *__restrict__
             }
     }
     box_fold(v, s_red);
-    if (threadIdx.x < 6) part[1 + 6 * blockIdx.x + threadIdx.x] = s_red[0][threadIdx.x];
+    if (threadIdx.x < 6) part[6 * blockIdx.x + threadIdx.x] = s_red[0][threadIdx.x];
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(part, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     for (int a = 0; a < 6; ++a) v[a] = a < 3 ? 0xffffffffu : 0u;
     for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
         for (int a = 0; a < 6; ++a) {
-            const uint32_t o = *(volatile uint32_t *)&part[1 + 6 * b + a];
+            const uint32_t o = *(volatile uint32_t *)&part[6 * b + a];
             v[a] = a < 3 ? min(v[a], o) : max(v[a], o);
         }
     box_fold(v, s_red);
@@ -224,7 +224,6 @@ __global__ void __launch_bounds__(256) box_geom_kernel(const float *__restrict__
             off_one[0] = 0;
             off_one[1] = n;
         }
-        *part = 0u;
     }
 }
 
@@ -1104,7 +1103,8 @@ cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, c
     }
     if (B == 1) {
         if ((e = sort_clear_u32(n, c->sort, st))) return e;
-        box_geom_kernel<<<box_blocks(n), 256, 0, st>>>(x, y, z, n, box, c->d_box, c->d_geom,
+        box_geom_kernel<<<box_blocks(n), 256, 0, st>>>(x, y, z, n, box, c->d_box,
+                                                       sort_zero_word(c->sort), c->d_geom,
                                                        c->d_off);
         note_launch();
         morton_one_kernel<<<morton_blocks(n, c->num_sms), 256, 0, st>>>(
@@ -1220,7 +1220,8 @@ cudaError_t octree_reduce(relearn_ctx *c, const int32_t *vac_de, cudaStream_t st
 // loads this library keeps it until the process exits. All calls on a device
 // share it and it keeps the previous call's contents, so calls whose GPU work
 // overlaps (different streams, no ordering between them) race on it. Every call
-// resets what has to start at zero.
+// zeroes the words it counts in (the head of the sort's scratch) before it counts, so
+// whatever the array holds at its start, a call that overlaps none gives the right order.
 // ---------------------------------------------------------------------------
 namespace rl {
 namespace {
@@ -1236,7 +1237,7 @@ constexpr size_t kOffStatus = kOffHist + 4 * kNoAllocSortWords;
 constexpr size_t kNoAllocBytes = kOffStatus + 4;
 // the regions must not overlap: the blocks' box words below the geometry, the geometry
 // below the sort's ping-pong buffers
-static_assert((1 + 6 * kBoxBlocks) * sizeof(uint32_t) <= kOffGeom, "box words overlap the geometry");
+static_assert(6 * kBoxBlocks * sizeof(uint32_t) <= kOffGeom, "box words overlap the geometry");
 static_assert(kOffGeom + sizeof(Geom) <= kOffCodesAlt, "geometry overlaps the sort buffers");
 static_assert(kOffHist % 8 == 0, "the sort's scratch must be 8-byte aligned");
 
@@ -1323,7 +1324,8 @@ extern "C" relearn_status relearn_morton_order_noalloc(int64_t n, const float *x
         return cudaGetLastError() == cudaSuccess ? RELEARN_OK : RELEARN_ERR_CUDA;
     }
     if (sort_clear_u32(n, ss, st) != cudaSuccess) return RELEARN_ERR_CUDA;
-    box_geom_kernel<<<box_blocks(n), 256, 0, st>>>(x, y, z, n, box, part, geom, nullptr);
+    box_geom_kernel<<<box_blocks(n), 256, 0, st>>>(x, y, z, n, box, part, sort_zero_word(ss),
+                                                   geom, nullptr);
     note_launch();
     morton_one_kernel<<<morton_blocks(n, d.num_sms), 256, 0, st>>>(x, y, z, n, geom, codes, perm,
                                                                    sort_counts(ss));

@@ -221,8 +221,9 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Scratch: the passes' digit counts, tickets and the abort flag, then two sets of tile
-// states, used in turn (each pass clears the next one's).
+// Scratch: the passes' digit counts, tickets, the abort flag and the word of
+// sort_zero_word, then two sets of tile states, used in turn (each pass clears the next
+// one's).
 constexpr int64_t kHead = kMaxPasses * kRadix + kMaxPasses + 8;
 
 template <typename K>
@@ -266,6 +267,10 @@ int64_t sort_blocks_needed(int64_t max_n) { return (max_n + kTile - 1) / kTile; 
 int64_t sort_scratch_words(int64_t blocks) { return kHead + 2 * kRadix * blocks; }
 
 uint32_t *sort_counts(SortScratch &s) { return reinterpret_cast<uint32_t *>(s.hist); }
+uint32_t *sort_zero_word(SortScratch &s)
+{
+    return sort_counts(s) + kMaxPasses * kRadix + kMaxPasses + 1;
+}
 
 cudaError_t sort_clear_u32(int64_t n, SortScratch &s, cudaStream_t st)
 {

@@ -25,3 +25,7 @@ def _run(tmp_path, program, sources=()):
 
 def test_sort_pass_ignores_tickets_past_its_grid(tmp_path):
     _run(tmp_path, "sort_tickets.cu")
+
+
+def test_noalloc_order_does_not_depend_on_what_its_scratch_holds(tmp_path):
+    _run(tmp_path, "noalloc_scratch.cu", ("sort.cu", "scan.cu"))
