@@ -239,6 +239,12 @@ relearn_status relearn_update_connectivity_typed(relearn_ctx *ctx, const relearn
  * the hook. Errors: INVALID_ARG for NULL. */
 relearn_status relearn_debug_stall_scan(relearn_ctx *ctx, int64_t tile);
 
+/* Testing hook: while on != 0, calls on this context take the kernels of large networks
+ * whatever the network's size, as they do where the GPU, or the part of it that the
+ * process may use, cannot place a cluster of 16 thread blocks. Results are the same.
+ * Errors: INVALID_ARG for NULL. */
+relearn_status relearn_debug_no_clusters(relearn_ctx *ctx, int32_t on);
+
 /* Deletion pass (Sec. III-A "Update of synapses", first sub-phase).
  *   retract_ax, retract_de  device int32[n] (>= 0): elements each neuron retracts.
  *   vac_ax, vac_de          device int32[n], in/out.

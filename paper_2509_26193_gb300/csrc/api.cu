@@ -276,8 +276,8 @@ relearn_status relearn_create_batched(relearn_ctx **out, int device, int64_t max
     A(scan.flags, scan_blocks + 3);
 #undef A
     if (e == cudaSuccess) {
-        for (auto init : {octree_init, search_init, synapses_init, length_init})
-            if (e == cudaSuccess) e = init();
+        c->clusters = octree_clusters() && search_clusters() && synapses_clusters() &&
+                      length_clusters();
         c->scan.max_blocks = scan_blocks;
         c->scan.status = c->d_status;
         c->scan.grid_cap = scan_grid_cap(c->num_sms);
@@ -506,6 +506,13 @@ relearn_status relearn_debug_stall_scan(relearn_ctx *c, int64_t tile)
 {
     if (!c) return RELEARN_ERR_INVALID_ARG;
     c->debug_stall_tile = tile < 0 ? -1 : tile;
+    return RELEARN_OK;
+}
+
+relearn_status relearn_debug_no_clusters(relearn_ctx *c, int32_t on)
+{
+    if (!c) return RELEARN_ERR_INVALID_ARG;
+    c->no_clusters = on != 0;
     return RELEARN_OK;
 }
 

@@ -54,6 +54,8 @@ struct SearchConst {
 struct relearn_ctx {
     int device = 0;
     int num_sms = 0;
+    bool clusters = false;    // clusters of 16 blocks can be placed (asked at creation)
+    bool no_clusters = false; // relearn_debug_no_clusters
     // resident blocks per SM: [2 * batched + diagnostics][union, split]
     int search_occ[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
     int split_occ[2][33] = {};  // split kernel blocks per SM, by network kind and capacity / 32
@@ -157,11 +159,12 @@ namespace rl {
 
 // Whether a context's passes over its neurons and synapses run as one cluster kernel each
 // (cluster.cuh): by its sizes and capacities, since the counts of searches and synapses
-// are known on the device only.
+// are known on the device only. Without clusters the general kernels serve every size.
 constexpr int64_t kSmallN = 40960, kSmallItems = 8 * kSmallN, kSmallBuildN = 32768;
+inline bool may_cluster(const relearn_ctx *c) { return c->clusters && !c->no_clusters; }
 inline bool small_network(const relearn_ctx *c)
 {
-    return c->n <= kSmallN && c->max_searches <= kSmallItems && c->max_synapses <= kSmallItems;
+    return may_cluster(c) && c->n <= kSmallN && c->max_searches <= kSmallItems && c->max_synapses <= kSmallItems;
 }
 
 // Blocks for a grid-stride loop over n items: enough to cover n, at most 32 per SM.
@@ -203,11 +206,12 @@ cudaError_t radix_sort_u64(uint64_t *keys, uint64_t *keys_alt, int32_t *vals, in
 int64_t sort_blocks_needed(int64_t max_n);
 int64_t sort_scratch_words(int64_t blocks);
 
-// Launch attributes of each file's cluster kernels on the current device.
-cudaError_t octree_init();
-cudaError_t search_init();
-cudaError_t synapses_init();
-cudaError_t length_init();
+// Whether each file's cluster kernels can run in the current context (also sets their
+// launch attributes there).
+bool octree_clusters();
+bool search_clusters();
+bool synapses_clusters();
+bool length_clusters();
 
 // octree.cu -----------------------------------------------------------------
 cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, const float *y,

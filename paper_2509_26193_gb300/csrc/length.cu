@@ -1117,7 +1117,7 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
     p.fam = c->d_fam;
     p.lsum = c->d_lsum;
     p.work = c->d_i32 + I32_WORK;
-    if (n <= kSmallLen) {
+    if (n <= kSmallLen && may_cluster(c)) {
         len_prepare_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(p);
         note_launch();
     } else {
@@ -1170,9 +1170,6 @@ cudaError_t length_backward(relearn_ctx *c, const int32_t *vac_ax, const int32_t
     return cudaGetLastError();
 }
 
-cudaError_t length_init()
-{
-    return cluster_form::allow(len_prepare_small_kernel);
-}
+bool length_clusters() { return cluster_form::placeable(len_prepare_small_kernel); }
 
 } // namespace rl

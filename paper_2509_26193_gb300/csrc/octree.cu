@@ -1091,7 +1091,7 @@ cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, c
     const unsigned gn = grid_for(n, 256, c->num_sms);
     const unsigned gb = (unsigned)((B + 255) / 256);
     int which = 0;
-    if (B == 1 && n <= kSmallBuildN) {
+    if (B == 1 && n <= kSmallBuildN && may_cluster(c)) {
         build_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
             MortonArgs{n, x, y, z, box, c->d_geom, c->d_codes, c->d_codes_alt, c->d_perm,
                        c->d_perm_alt},
@@ -1158,12 +1158,10 @@ cudaError_t octree_build(relearn_ctx *c, int64_t n, int32_t B, const float *x, c
     return cudaGetLastError();
 }
 
-cudaError_t octree_init()
+bool octree_clusters()
 {
-    cudaError_t e;
-    if ((e = cluster_form::allow(build_small_kernel))) return e;
-    if ((e = cluster_form::allow(morton_small_kernel))) return e;
-    return cluster_form::allow(reduce_small_kernel);
+    return cluster_form::placeable(build_small_kernel) &&
+           cluster_form::placeable(reduce_small_kernel);
 }
 
 cudaError_t octree_reduce(relearn_ctx *c, const int32_t *vac_de, cudaStream_t st)
@@ -1264,7 +1262,6 @@ relearn_status noalloc_setup(int dev, NoAllocDevice *out)
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return RELEARN_ERR_CUDA;
-        if (octree_init() != cudaSuccess) return RELEARN_ERR_CUDA;
         g_noalloc_sms[dev] = sms > 0 ? sms : 1;
     }
     out->base = static_cast<unsigned char *>(p);
@@ -1317,7 +1314,9 @@ extern "C" relearn_status relearn_morton_order_noalloc(int64_t n, const float *x
             box.lo[a] = box_lo3[a];
             box.hi[a] = box_hi3[a];
         }
-    if (n <= kSmallN) {
+    // asked on every call: the answer and the attribute belong to the context, which a
+    // device reset replaces
+    if (n <= kSmallN && cluster_form::placeable(morton_small_kernel)) {
         morton_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
             MortonArgs{n, x, y, z, box, geom, codes, codes_alt, perm, perm_alt});
         note_launch();

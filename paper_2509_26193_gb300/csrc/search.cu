@@ -1149,7 +1149,7 @@ cudaError_t search_constants(relearn_ctx *c, const relearn_params &p, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t search_init() { return cluster_form::allow(query_small_kernel); }
+bool search_clusters() { return cluster_form::placeable(query_small_kernel); }
 
 cudaError_t search_prepare(relearn_ctx *c, const relearn_params &p, const int32_t *vac_ax,
                            cudaStream_t st)

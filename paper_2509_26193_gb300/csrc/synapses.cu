@@ -821,12 +821,11 @@ cudaError_t canonicalise_store(relearn_ctx *c, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t synapses_init()
+bool synapses_clusters()
 {
-    cudaError_t e;
-    if ((e = cluster_form::allow(accept_apply_small_kernel))) return e;
-    if ((e = cluster_form::allow(delete_small_kernel))) return e;
-    return cluster_form::allow(deliver_small_kernel);
+    return cluster_form::placeable(accept_apply_small_kernel) &&
+           cluster_form::placeable(delete_small_kernel) &&
+           cluster_form::placeable(deliver_small_kernel);
 }
 
 cudaError_t accept_apply_small(relearn_ctx *c, const relearn_params &p, int32_t *vac_ax,

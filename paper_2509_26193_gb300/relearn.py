@@ -74,6 +74,7 @@ _SIGS = {
     "relearn_deliver_spikes": [_P, _P, _P, _P],
     "relearn_mean_length": [_P, ctypes.POINTER(relearn_params), _P, _P, _P, _P, _P],
     "relearn_debug_stall_scan": [_P, ctypes.c_int64],
+    "relearn_debug_no_clusters": [_P, ctypes.c_int32],
     "relearn_update_connectivity_typed": [_P, ctypes.POINTER(relearn_params), _P, _P, _P, _P,
                                           ctypes.POINTER(relearn_update_stats), _P],
     "relearn_mean_length_backward": [_P, _P, _P, _P, _P, _P, _P, _P, _P],
@@ -270,6 +271,13 @@ def relearn_debug_stall_scan(ctx, tile):
     nothing, so that update's bounded waits run out (RELEARN_ERR_TIMEOUT)."""
     _raise(ctx, lib().relearn_debug_stall_scan(ctx.handle, int(tile)),
            "relearn_debug_stall_scan")
+
+
+def relearn_debug_no_clusters(ctx, on):
+    """Testing hook: while on, calls on ctx run no cluster kernels, as on a GPU (or a part
+    of one) that cannot place a cluster of 16 blocks."""
+    _raise(ctx, lib().relearn_debug_no_clusters(ctx.handle, int(bool(on))),
+           "relearn_debug_no_clusters")
 
 
 def relearn_build_octree_batch(ctx, offsets, x, y, z, vac_de=None, stream=None):

@@ -74,5 +74,9 @@ int main()
     for (int64_t n : {700, 40960, 40961, 300000})
         for (int fill : {-1, 0, 1, 0xFF, 0x5A})
             if (!check(n, fill)) return 1;
+    // a context made anew after a reset of the device (with nothing in flight) is served too
+    if (cudaDeviceReset() != cudaSuccess) return 1;
+    for (int64_t n : {700, 40961})
+        if (!check(n, -1)) return 1;
     return 0;
 }
