@@ -510,6 +510,87 @@ __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ 
 #define CLUSTER_STRIDE(i, n)                                                                      \
     for (int64_t i = cluster_form::first(); i < (n); i += cluster_form::kStride)
 
+// Rows longer than kLongRow (a hub's requests or synapses) are not ranked by counting:
+// that takes the square of the length, which 16 SMs take several times as long over as the
+// general kernels' 152. Instead each run of kRun entries is sorted (one block per run, in
+// shared memory), and an entry's place is its place in its own run plus a binary search in
+// each other one. One target taking every request of 20,000 / 40,000 neurons, 1,000 /
+// 2,000 vacancies: update 4.07 / 15.6 ms by counting, 0.30 / 0.95 here, 1.9 / 3.7 by the
+// general kernels; canonical order with an in-degree of 20,000: 840 us, 197, 443. The flag
+// any_long (set by the scans of the row lengths) keeps the passes out of networks without
+// such rows.
+constexpr int32_t kLongRow = 256, kRun = cluster_form::kThreads;
+
+// Sorts every run of kRun entries of the rows ptr[i] .. ptr[i + 1] longer than kLongRow (at
+// most kSmallItems entries in all), by keys of type K below the largest of K: load(i) is
+// entry i's key, store(i, key) puts it back. Called by the whole cluster; a barrier has to
+// follow.
+template <class K, class Load, class Store>
+__device__ __forceinline__ void sort_runs(const int32_t *ptr, int64_t n, K largest, Load load,
+                                          Store store)
+{
+    namespace cf = cluster_form;
+    __shared__ K s_key[kRun];
+    __shared__ int32_t s_row[kSmallItems / kLongRow];
+    __shared__ int32_t s_rows;
+    const int t = threadIdx.x, rank = (int)cooperative_groups::this_cluster().block_rank();
+    if (t == 0) s_rows = 0;
+    __syncthreads();
+    for (int64_t i = t; i < n; i += cf::kThreads) // every block lists every long row
+        if (ptr[i + 1] - ptr[i] > kLongRow) s_row[atomicAdd(&s_rows, 1)] = (int32_t)i;
+    __syncthreads();
+    for (int q = 0; q < s_rows; ++q) {
+        const int32_t b = ptr[s_row[q]], e = ptr[s_row[q] + 1];
+        for (int32_t s = b; s < e; s += kRun) {
+            if ((s / kRun) % cf::kBlocks != rank) continue; // the same block for every list order
+            s_key[t] = s + t < e ? load(s + t) : largest;
+            __syncthreads();
+            for (int k = 2; k <= kRun; k <<= 1) // bitonic sort
+                for (int j = k >> 1; j; j >>= 1) {
+                    const int p = t ^ j;
+                    if (p > t) {
+                        const K x = s_key[t], y = s_key[p];
+                        if ((x > y) == ((t & k) == 0)) {
+                            s_key[t] = y;
+                            s_key[p] = x;
+                        }
+                    }
+                    __syncthreads();
+                }
+            if (s + t < e) store(s + t, s_key[t]);
+            __syncthreads();
+        }
+    }
+}
+
+// How many entries of the row b .. e (its runs sorted by keys) come before entry r, whose
+// key is given: smaller keys, and of equal ones those at smaller places. r = -1: how many
+// keys are smaller.
+template <class K>
+__device__ __forceinline__ int32_t place_in_runs(const K *keys, int32_t b, int32_t e, K key,
+                                                 int64_t r)
+{
+    int32_t place = 0;
+    for (int32_t s = b; s < e; s += kRun) {
+        const int32_t end = min(s + kRun, e);
+        int32_t lo = s, hi = end;
+        if (r >= s && r < end) {
+            place += (int32_t)r - s;
+            continue;
+        }
+        const bool ties = end <= r;
+        while (lo < hi) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (keys[mid] < key || (ties && keys[mid] == key))
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        place += lo - s;
+    }
+    return place;
+}
+
 struct StoreArgs {
     int64_t n, max_synapses;
     int32_t *d_nsyn;
@@ -534,11 +615,20 @@ struct AcceptArgs {
     uint32_t *prio;
     int32_t *tcnt, *toff;
     uint64_t *bucket;
+    int32_t *any_long;
     uint8_t *acc;
     int64_t *declined, *formed;
     int32_t *vac_ax, *vac_de;
     const uint8_t *type;
 };
+
+// As accepted, for a request of a long row (runs sorted).
+__device__ __forceinline__ bool accepted_long(int64_t r, int32_t t, const AcceptArgs &a)
+{
+    const int32_t v = max(a.vac_de[t], 0), b = a.toff[t], e = a.toff[t + 1];
+    if (e - b <= v) return true;
+    return v > 0 && place_in_runs(a.bucket, b, e, request_key(a.prio[r], r), -1) < v;
+}
 
 // Acceptance and apply of an update.
 __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
@@ -549,7 +639,10 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     const int64_t base = *st.d_nsyn;
     const bool failed = *(volatile int32_t *)a.status != 0; // an earlier kernel's error
     CLUSTER_STRIDE(i, st.n + 1) a.tcnt[i] = 0;
-    if (cf::first() == 0) *a.declined = 0;
+    if (cf::first() == 0) {
+        *a.declined = 0;
+        *a.any_long = 0;
+    }
     cf::sync();
     CLUSTER_STRIDE(r, Q)
     {
@@ -561,10 +654,13 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     }
     cf::sync();
     auto count = [&](int64_t i) { return cf::I32{a.tcnt[i]}; };
-    cf::scan<cf::I32>(st.n + 1, count, count, [&](int64_t i, cf::I32 prefix, cf::I32, cf::I32) {
-        a.toff[i] = prefix.v;
-    });
+    cf::scan<cf::I32>(st.n + 1, count, count,
+                      [&](int64_t i, cf::I32 prefix, cf::I32 requests, cf::I32) {
+                          a.toff[i] = prefix.v;
+                          if (requests.v > kLongRow) *a.any_long = 1;
+                      });
     cf::sync();
+    const bool any_long = *(volatile int32_t *)a.any_long != 0;
     CLUSTER_STRIDE(r, Q)
     {
         const int32_t t = a.req_tgt[r];
@@ -572,13 +668,21 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
             a.bucket[a.toff[t] + atomicSub(&a.tcnt[t], 1) - 1] = request_key(a.prio[r], r);
     }
     cf::sync();
+    if (any_long) {
+        sort_runs(a.toff, st.n, ~uint64_t(0), [&](int64_t i) { return a.bucket[i]; },
+                  [&](int64_t i, uint64_t key) { a.bucket[i] = key; });
+        cf::sync();
+    }
     int64_t dec = 0;
     // every decision is made before the first vacancy changes (the scan's barrier)
     const cf::I32 formed = cf::scan<cf::I32>(
         Q,
         [&](int64_t r) {
             const int32_t t = a.req_tgt[r];
-            const bool ok = t >= 0 && accepted(r, t, a.prio, a.toff, a.bucket, a.vac_de);
+            const bool ok =
+                t >= 0 && (any_long && a.toff[t + 1] - a.toff[t] > kLongRow
+                               ? accepted_long(r, t, a)
+                               : accepted(r, t, a.prio, a.toff, a.bucket, a.vac_de));
             dec += t >= 0 && !ok ? 1 : 0;
             a.acc[r] = ok ? 1 : 0;
             return cf::I32{ok ? 1 : 0};
@@ -612,7 +716,7 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
 struct DeleteArgs {
     bool canonical; // the views below are those of the store
     int32_t *out_cnt, *in_cnt, *out_ptr, *in_ptr;
-    int32_t *row_src, *row_tgt, *row_sign, *row_k, *in_syn;
+    int32_t *row_src, *row_tgt, *row_sign, *row_k, *in_syn, *any_long;
     const int32_t *retract_ax, *retract_de;
     int32_t *vac_ax, *vac_de, *need_ax, *need_de;
     uint32_t *prio_ax, *prio_de;
@@ -629,6 +733,7 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     const int64_t n = st.n, m = *st.d_nsyn;
     if (!a.canonical) {
         CLUSTER_STRIDE(i, n + 1) a.out_cnt[i] = a.in_cnt[i] = 0;
+        if (cf::first() == 0) *a.any_long = 0;
         cf::sync();
         CLUSTER_STRIDE(k, m)
         {
@@ -638,11 +743,13 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
         cf::sync();
         auto counts = [&](int64_t i) { return cf::I64x2{a.out_cnt[i], a.in_cnt[i]}; };
         cf::scan<cf::I64x2>(n + 1, counts, counts,
-                            [&](int64_t i, cf::I64x2 prefix, cf::I64x2, cf::I64x2) {
+                            [&](int64_t i, cf::I64x2 prefix, cf::I64x2 degree, cf::I64x2) {
                                 a.out_ptr[i] = (int32_t)prefix.a;
                                 a.in_ptr[i] = (int32_t)prefix.b;
+                                if (degree.a > kLongRow || degree.b > kLongRow) *a.any_long = 1;
                             });
         cf::sync();
+        const bool any_long = *(volatile int32_t *)a.any_long != 0;
         CLUSTER_STRIDE(k, m)
         {
             const int32_t s = st.src[k];
@@ -652,9 +759,21 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
             a.row_sign[r] = st.sign[k];
         }
         cf::sync();
+        if (any_long) { // by (target, sign): the sign moves with its record
+            sort_runs(a.out_ptr, n, 0x7fffffff,
+                      [&](int64_t i) { return 2 * a.row_tgt[i] + (a.row_sign[i] > 0 ? 1 : 0); },
+                      [&](int64_t i, int32_t key) {
+                          a.row_tgt[i] = key >> 1;
+                          a.row_sign[i] = key & 1 ? 1 : -1;
+                      });
+            cf::sync();
+        }
         CLUSTER_STRIDE(r, m)
         {
-            const int32_t w = row_place(r, a.row_src, a.row_tgt, a.out_ptr);
+            const int32_t s = a.row_src[r], b = a.out_ptr[s], e = a.out_ptr[s + 1];
+            const int32_t w = any_long && e - b > kLongRow
+                                  ? b + place_in_runs(a.row_tgt, b, e, a.row_tgt[r], r)
+                                  : row_place(r, a.row_src, a.row_tgt, a.out_ptr);
             st.src[w] = a.row_src[r];
             st.tgt[w] = a.row_tgt[r];
             st.sign[w] = (int8_t)a.row_sign[r];
@@ -666,7 +785,18 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
             a.row_k[a.in_ptr[t] + atomicSub(&a.in_cnt[t], 1) - 1] = (int32_t)k;
         }
         cf::sync();
-        CLUSTER_STRIDE(r, m) a.in_syn[in_place(r, a.row_k, st.tgt, a.in_ptr)] = a.row_k[r];
+        if (any_long) {
+            sort_runs(a.in_ptr, n, 0x7fffffff, [&](int64_t i) { return a.row_k[i]; },
+                      [&](int64_t i, int32_t k) { a.row_k[i] = k; });
+            cf::sync();
+        }
+        CLUSTER_STRIDE(r, m)
+        {
+            const int32_t k = a.row_k[r], t = st.tgt[k], b = a.in_ptr[t], e = a.in_ptr[t + 1];
+            a.in_syn[any_long && e - b > kLongRow
+                         ? b + place_in_runs(a.row_k, b, e, k, r)
+                         : in_place(r, a.row_k, st.tgt, a.in_ptr)] = k;
+        }
         cf::sync();
     }
     CLUSTER_STRIDE(i, n)
@@ -841,6 +971,7 @@ cudaError_t accept_apply_small(relearn_ctx *c, const relearn_params &p, int32_t 
     a.tcnt = c->d_tcnt;
     a.toff = c->d_toff;
     a.bucket = c->d_bucket;
+    a.any_long = c->d_i32 + I32_LONG;
     a.acc = c->d_req_acc;
     a.declined = c->d_i64 + I64_DECLINED;
     a.formed = c->d_i64 + I64_FORMED;
@@ -901,6 +1032,7 @@ cudaError_t delete_synapses(relearn_ctx *c, const relearn_params &p, const int32
         a.row_tgt = reinterpret_cast<int32_t *>(c->d_key32);
         a.row_k = reinterpret_cast<int32_t *>(c->d_key32_alt);
         a.in_syn = c->d_in_syn;
+        a.any_long = c->d_i32 + I32_LONG;
         a.retract_ax = retract_ax;
         a.retract_de = retract_de;
         a.vac_ax = vac_ax;
