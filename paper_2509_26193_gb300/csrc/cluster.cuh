@@ -10,7 +10,10 @@
 // theta 0.5; us, general kernels -> cluster kernels of 8 x 1024, 16 x 1024 and 16 x 512
 // threads): 1,000 neurons 402 -> 238 / 253 / 217, 8,000 533 -> 358 / 344 / 328, 16,000
 // 634 -> 516 / 479 / 476, 32,000 853 -> 883 / 759 / 797, 50,000 1156 -> 1366 / 1162 / 1218:
-// hence 16 x 512, up to kSmallN = 40,960 neurons (internal.h).
+// hence 16 x 512, up to kSmallN = 40,960 neurons (internal.h). Replayed from a graph,
+// without launch gaps (an update and a full deletion): 131 -> 87, 146 -> 109 (4,000), 178 ->
+// 149, 252 -> 232, 399 -> 387, 437 -> 496 (40,000); deliveries then choose for themselves
+// (deliver_small in synapses.cu).
 #pragma once
 
 #include <cooperative_groups.h>

@@ -416,51 +416,56 @@ __global__ void shrink_store_kernel(int32_t *d_nsyn, const int64_t *d_kept, int6
 
 // ---------------------------------------------------------------- spikes
 // input[t] += sign for every synapse s -> t of a spiking source (input zeroed first).
-// A thread takes four neighbouring synapses: each synapse is a chain of dependent reads
+// A thread takes W neighbouring synapses: each synapse is a chain of dependent reads
 // (source, its spike or rate, target, atomic), and four chains in flight per thread wait
 // for them together (1.8 million synapses, 5 % firing, with the zeroing of the inputs:
-// 12.4 -> 10.9 us a call, of which about 9 are the two launches).
-struct Four {
-    int32_t v[4];
+// 12.4 -> 10.9 us a call, of which about 9 are the two launches). A store that the
+// resident threads cover with one synapse each takes W = 1 (see deliver_width).
+template <int W>
+struct Some {
+    int32_t v[W];
 };
 
-// Entries 4 q .. 4 q + 3 of a store array (16-byte aligned), `fill` past its end m.
-__device__ __forceinline__ Four four_of(const int32_t *__restrict__ a, int64_t q, int64_t m,
-                                        int32_t fill)
+// Entries W q .. W q + W - 1 of a store array (16-byte aligned), `fill` past its end m.
+template <int W>
+__device__ __forceinline__ Some<W> some_of(const int32_t *__restrict__ a, int64_t q, int64_t m,
+                                           int32_t fill)
 {
-    Four f;
-    if (4 * q + 4 <= m) {
+    Some<W> f;
+    if (W == 4 && 4 * q + 4 <= m) {
         const int4 w = __ldg(reinterpret_cast<const int4 *>(a) + q);
         f.v[0] = w.x;
-        f.v[1] = w.y;
-        f.v[2] = w.z;
-        f.v[3] = w.w;
+        f.v[1 % W] = w.y;
+        f.v[2 % W] = w.z;
+        f.v[3 % W] = w.w;
     } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) f.v[k] = 4 * q + k < m ? a[4 * q + k] : fill;
+        for (int k = 0; k < W; ++k) f.v[k] = W * q + k < m ? a[W * q + k] : fill;
     }
     return f;
 }
 
-__device__ __forceinline__ void four_spikes(int64_t q, int64_t m, const int32_t *src,
+template <int W>
+__device__ __forceinline__ void some_spikes(int64_t q, int64_t m, const int32_t *src,
                                             const int32_t *tgt, const int8_t *sign,
                                             const uint8_t *spiked, int32_t *input)
 {
-    const Four s = four_of(src, q, m, -1);
-    uint8_t on[4];
+    const Some<W> s = some_of<W>(src, q, m, -1);
+    uint8_t on[W];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) on[k] = s.v[k] >= 0 ? spiked[s.v[k]] : 0;
+    for (int k = 0; k < W; ++k) on[k] = s.v[k] >= 0 ? spiked[s.v[k]] : 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (on[k]) atomicAdd(&input[tgt[4 * q + k]], (int32_t)sign[4 * q + k]);
+    for (int k = 0; k < W; ++k)
+        if (on[k]) atomicAdd(&input[tgt[W * q + k]], (int32_t)sign[W * q + k]);
 }
 
+template <int W>
 __global__ void spikes_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
                               const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
                               const uint8_t *__restrict__ spiked, int32_t *__restrict__ input)
 {
     const int64_t m = *d_nsyn;
-    GRID_STRIDE(q, (m + 3) / 4) four_spikes(q, m, src, tgt, sign, spiked, input);
+    GRID_STRIDE(q, (m + W - 1) / W) some_spikes<W>(q, m, src, tgt, sign, spiked, input);
 }
 
 // Firing-rate delivery (Sec. IV-B): the receiver t decides once per step and per
@@ -477,30 +482,32 @@ __device__ __forceinline__ bool rate_fires(int32_t s, int32_t t, float rate, uin
     return rate > 0.0f && w < __float2uint_ru(__fmul_rn(rate, 4294967296.0f)); // NaN: never
 }
 
-__device__ __forceinline__ void four_rates(int64_t q, int64_t m, const int32_t *src,
+template <int W>
+__device__ __forceinline__ void some_rates(int64_t q, int64_t m, const int32_t *src,
                                            const int32_t *tgt, const int8_t *sign,
                                            const float *rate, uint64_t seed, uint32_t step,
                                            int32_t *input)
 {
-    const Four s = four_of(src, q, m, -1), t = four_of(tgt, q, m, 0);
-    float r[4];
+    const Some<W> s = some_of<W>(src, q, m, -1), t = some_of<W>(tgt, q, m, 0);
+    float r[W];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) r[k] = s.v[k] >= 0 ? rate[s.v[k]] : 0.0f;
+    for (int k = 0; k < W; ++k) r[k] = s.v[k] >= 0 ? rate[s.v[k]] : 0.0f;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < W; ++k)
         if (rate_fires(s.v[k], t.v[k], r[k], seed, step))
-            atomicAdd(&input[t.v[k]], (int32_t)sign[4 * q + k]);
+            atomicAdd(&input[t.v[k]], (int32_t)sign[W * q + k]);
 }
 
 // As spikes_kernel (1.8 million synapses 19.7 -> 14.4 us a call, 3.4 million 31.0 -> 18.6;
 // one, two or four synapses per thread are the same here: the generator bounds it).
+template <int W>
 __global__ void rates_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
                              const int32_t *__restrict__ tgt, const int8_t *__restrict__ sign,
                              const float *__restrict__ rate, uint64_t seed, uint32_t step,
                              int32_t *__restrict__ input)
 {
     const int64_t m = *d_nsyn;
-    GRID_STRIDE(q, (m + 3) / 4) four_rates(q, m, src, tgt, sign, rate, seed, step, input);
+    GRID_STRIDE(q, (m + W - 1) / W) some_rates<W>(q, m, src, tgt, sign, rate, seed, step, input);
 }
 
 // ---------------------------------------------------------------- small networks
@@ -850,9 +857,8 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
 }
 
 // input = 0, then as spikes_kernel (spiked given) or rates_kernel: one launch instead of a
-// memset and a kernel (a spike and a rate delivery called in turn, 5,000 to 40,000 neurons:
-// 20.6 -> 16.6 us; replayed from a graph, which has no launch gaps to save, 8.3 to 10.3
-// before, 10.3 to 12.4 now).
+// memset and a kernel (called directly, 4,000 to 40,000 neurons: spikes 10.2 -> 8.3 us,
+// rates 10.4 -> 8.6; for graphs see deliver_small).
 __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     __launch_bounds__(cluster_form::kThreads)
     deliver_small_kernel(const int32_t *d_nsyn, const int32_t *__restrict__ src,
@@ -867,10 +873,42 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     CLUSTER_STRIDE(q, (m + 3) / 4)
     {
         if (spiked)
-            four_spikes(q, m, src, tgt, sign, spiked, input);
+            some_spikes<4>(q, m, src, tgt, sign, spiked, input);
         else
-            four_rates(q, m, src, tgt, sign, rate, seed, step, input);
+            some_rates<4>(q, m, src, tgt, sign, rate, seed, step, input);
     }
+}
+
+} // namespace
+
+namespace {
+
+// Synapses per thread of the general delivery kernels, by the store's capacity: up to one
+// and a half per resident thread, four to a thread leave the chip idle (in a graph of 40
+// calls, us a call, spikes / rates, one -> four per thread: 32,904 3.2 / 3.2 -> 3.6 / 4.1,
+// 400,946 3.5 / 3.7 -> 3.7 / 4.4, 800,072 4.4 / 4.5 -> 3.8 / 4.7, 1,601,212 5.9 / 6.3 ->
+// 4.1 / 5.8, 4,186,726 8.3 / 9.9 -> 5.8 / 9.2).
+int deliver_width(const relearn_ctx *c)
+{
+    return c->max_synapses <= 3072 * (int64_t)c->num_sms ? 1 : 4;
+}
+
+// Whether a delivery runs as one cluster kernel (see deliver_small_kernel): called
+// directly, it saves a launch. Replayed from a graph it saves none, and the general form
+// spreads over the whole GPU; only where the inputs take at most 4 KB is the general form's
+// zeroing node slow (a graph of 40 calls, us a call, spikes / rates, cluster and general:
+// 1,000 neurons 2.9 / 3.7 and 6.2 / 6.2, 2,000 3.0 / 3.6 and 3.1 / 3.1, 16,000 3.2 / 4.0 and
+// 3.2 / 3.2, 40,000 4.4 / 5.7 and 3.3 / 3.2).
+bool deliver_small(const relearn_ctx *c, cudaStream_t st)
+{
+    if (!small_network(c)) return false;
+    if (c->n <= 1024) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError(); // the launch reports what is wrong with the stream
+        return true;
+    }
+    return cs == cudaStreamCaptureStatusNone;
 }
 
 } // namespace
@@ -878,7 +916,7 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
 cudaError_t deliver_rates(relearn_ctx *c, const float *rate, uint64_t seed, uint32_t step,
                           int32_t *input, cudaStream_t st)
 {
-    if (small_network(c)) {
+    if (deliver_small(c, st)) {
         deliver_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
             c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, nullptr, rate, seed, step, c->n,
             input);
@@ -887,8 +925,11 @@ cudaError_t deliver_rates(relearn_ctx *c, const float *rate, uint64_t seed, uint
     }
     cudaError_t e;
     if ((e = cudaMemsetAsync(input, 0, c->n * sizeof(int32_t), st))) return e;
-    rates_kernel<<<grid_for((c->max_synapses + 3) / 4, 256, c->num_sms), 256, 0, st>>>(
-        c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, rate, seed, step, input);
+    const int w = deliver_width(c);
+    (w == 1 ? rates_kernel<1> : rates_kernel<4>)
+        <<<grid_for((c->max_synapses + w - 1) / w, 256, c->num_sms), 256, 0, st>>>(
+            c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, rate, seed, step,
+            input);
     note_launch();
     return cudaGetLastError();
 }
@@ -1130,7 +1171,7 @@ cudaError_t merge_type(relearn_ctx *c, const int32_t *part, const uint8_t *type,
 cudaError_t deliver_spikes(relearn_ctx *c, const uint8_t *spiked, int32_t *input,
                            cudaStream_t st)
 {
-    if (small_network(c)) {
+    if (deliver_small(c, st)) {
         deliver_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(
             c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, spiked, nullptr, 0, 0, c->n,
             input);
@@ -1139,8 +1180,10 @@ cudaError_t deliver_spikes(relearn_ctx *c, const uint8_t *spiked, int32_t *input
     }
     cudaError_t e;
     if ((e = cudaMemsetAsync(input, 0, c->n * sizeof(int32_t), st))) return e;
-    spikes_kernel<<<grid_for((c->max_synapses + 3) / 4, 256, c->num_sms), 256, 0, st>>>(
-        c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, spiked, input);
+    const int w = deliver_width(c);
+    (w == 1 ? spikes_kernel<1> : spikes_kernel<4>)
+        <<<grid_for((c->max_synapses + w - 1) / w, 256, c->num_sms), 256, 0, st>>>(
+            c->d_i32 + I32_NSYN, c->d_syn_src, c->d_syn_tgt, c->d_syn_sign, spiked, input);
     note_launch();
     return cudaGetLastError();
 }
