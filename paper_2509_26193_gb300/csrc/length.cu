@@ -50,7 +50,10 @@ struct LenArgs {
     const int32_t *__restrict__ act_src;
     const int32_t *__restrict__ leaf_of;
     const int32_t *__restrict__ vac_ax;
+    int64_t n;              // neurons
     const int64_t *d_total; // active sources
+    int32_t *redo;          // groups left to redo_kernel: their number, its work counter
+    int32_t *redo_list;     // [n] which
     int64_t *evals_total;   // candidates visited (both passes)
     const SearchConst *sc;
     float4 *state;  // [n] per Morton position
@@ -325,7 +328,7 @@ __device__ __noinline__ void walk_pending(const LenArgs &a, const Src &s, uint2 
         sums[0] = __fsub_rn(f.s, f.sc);
         sums[1] = __fsub_rn(f.a, f.ac);
         sums[2] = __fsub_rn(f.b, f.bc);
-        sums[3] = 0.0f;
+        sums[3] = f.dmin2;
     }
     __syncwarp();
 }
@@ -548,9 +551,10 @@ struct GroupWalk {
     }
 };
 
-// The chunk's sums of this lane's source.
+// The chunk's sums of this lane's source (kNear: and its nearest D).
+template <bool kNear>
 __device__ __forceinline__ void fwd_chunk(const GroupShared *g, int n, const Src &src, float k2,
-                                          FwdSums &f)
+                                          FwdSums &f, float &nearest)
 {
     const uint32_t bit = 1u << (threadIdx.x & 31);
     const Pair xx = pack2(src.x.x, src.x.x), yy = pack2(src.x.y, src.x.y),
@@ -573,6 +577,10 @@ __device__ __forceinline__ void fwd_chunk(const GroupShared *g, int n, const Src
         f.s.add(at);
         f.a.add(mul2(at, pack2(sqrt_approx(D0), sqrt_approx(D1))));
         f.b.add(mul2(at, D));
+        if constexpr (kNear) {
+            if (on0) nearest = fminf(nearest, D0);
+            if (on1) nearest = fminf(nearest, D1);
+        }
     }
 }
 
@@ -652,6 +660,167 @@ __device__ __forceinline__ void bwd_chunk(const GroupShared *g, int n, const Src
     }
 }
 
+// One walk of a group by this warp, the sub-th of wpg that share it, with what each pass
+// adds up of the entries: the forward sums, these and the nearest D, or the adjoint.
+// members: the lanes whose sources take part, at least one.
+enum Pass { kSums, kNearSums, kAdjoint };
+template <Pass kPass>
+__device__ __forceinline__ void group_pass(const LenArgs &a, GroupWalk &w, const Src &s,
+                                           uint32_t members, int sub, int wpg, float k2,
+                                           float two_s2, FwdSums &f, BwdSums &b, float &nearest,
+                                           int64_t &evals)
+{
+    w.start(members, s.x, s.self);
+    if (wpg > 1) { // a pending list long enough to share out (at most 140 nodes)
+        while (w.top - w.base > 0 && w.top - w.base < 8 * wpg && w.top <= 72 &&
+               w.outc < kEntries - 64)
+            w.expand<true>();
+        w.take_share(sub, wpg);
+    }
+    for (;;) {
+        while (w.outc < kLenChunk && w.top > 0) {
+            if (w.top > kPend - 64 - kLenChunk) { // not reached by ordinary trees
+                const uint2 it = w.s->pend[--w.top];
+                float part[4];
+                walk_pending<kPass == kAdjoint>(a, s, it, w.thr0, k2, two_s2, part, evals);
+                if constexpr (kPass == kAdjoint) {
+                    b.cov.add_one(part[0]);
+                    b.gx.add_one(part[1]);
+                    b.gy.add_one(part[2]);
+                    b.gz.add_one(part[3]);
+                } else {
+                    f.s.add_one(part[0]);
+                    f.a.add_one(part[1]);
+                    f.b.add_one(part[2]);
+                    if constexpr (kPass == kNearSums) nearest = fminf(nearest, part[3]);
+                }
+            } else {
+                w.expand<false>();
+            }
+        }
+        const int n = min(w.outc, kLenChunk);
+        if (n == 0) break;
+        uint32_t kids;
+        const uint32_t tests = w.gather(n, kids, evals);
+        if (tests) w.resolve(tests, kids, s.x, evals);
+        if constexpr (kPass == kAdjoint)
+            bwd_chunk(w.s, n, s, k2, two_s2, a.G, b);
+        else
+            fwd_chunk<kPass == kNearSums>(w.s, n, s, k2, f, nearest);
+        __syncwarp(); // the chunk is overwritten next
+    }
+}
+
+using BlockSums = double[kGroupWarps][3][32];
+
+// Warps that share a group (see above for the line).
+__device__ __forceinline__ int warps_per_group(int32_t groups)
+{
+    int wpg = kGroupWarps;
+    while (wpg > 1 && (int64_t)groups * wpg > 2 * (int64_t)gridDim.x * kGroupWarps) wpg >>= 1;
+    return wpg;
+}
+
+// Takes the next of `count` groups for this warp (or, shared by wpg warps each, the next
+// kGroupWarps / wpg groups for the block, the last of them possibly past the count). False:
+// none left.
+__device__ __forceinline__ bool next_group(int32_t *work, int32_t count, int wpg, int32_t &s_next,
+                                           int32_t &at)
+{
+    if (wpg == 1) {
+        if ((threadIdx.x & 31) == 0) at = atomicAdd(work, 1);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        return at < count;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = atomicAdd(work, kGroupWarps / wpg);
+    __syncthreads();
+    at = s_next + (int32_t)(threadIdx.x >> 5) / wpg;
+    return s_next < count;
+}
+
+// Lanes that take no part (on: this one does) follow a lane that does.
+__device__ __forceinline__ void follow(uint32_t members, bool on, float3 &x)
+{
+    const int f = __ffs(members) - 1;
+    const float mx = __shfl_sync(0xffffffffu, x.x, f), my = __shfl_sync(0xffffffffu, x.y, f),
+                mz = __shfl_sync(0xffffffffu, x.z, f);
+    if (!on) x = make_float3(mx, my, mz);
+}
+
+// A source without a finite position has no finite distance and is left out.
+__device__ __forceinline__ bool finite_at(float4 p)
+{
+    return fabsf(p.x) + fabsf(p.y) + fabsf(p.z) < __int_as_float(0x7f800000);
+}
+
+// A source's state from its sums, and its share of the mean's numerator and denominator.
+__device__ __forceinline__ void finish_source(const LenArgs &a, int32_t sp, int32_t i, double S,
+                                              double sa, double sb, float k2sh, double &my0,
+                                              double &my1)
+{
+    float4 st = make_float4(0.f, 0.f, 0.f, k2sh);
+    if (S > 0.0) {
+        const double l = sa / S;
+        st.x = (float)l;
+        st.y = (float)(sb / S);
+        st.z = (float)(1.0 / S);
+        const double m = (double)a.vac_ax[i];
+        my0 += m * l;
+        my1 += m;
+    }
+    a.state[sp] = st;
+}
+
+__device__ __forceinline__ void add_totals(const LenArgs &a, double my0, double my1,
+                                           int64_t my_evals)
+{
+    for (int o = 16; o; o >>= 1) {
+        my0 += __shfl_xor_sync(0xffffffffu, my0, o);
+        my1 += __shfl_xor_sync(0xffffffffu, my1, o);
+        my_evals += __shfl_xor_sync(0xffffffffu, my_evals, o);
+    }
+    if ((threadIdx.x & 31) != 0) return;
+    if (my_evals)
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.evals_total),
+                  (unsigned long long)my_evals);
+    if (my1 > 0.0) {
+        atomicAdd(&a.lsum[0], my0);
+        atomicAdd(&a.lsum[1], my1);
+    }
+}
+
+// Sources whose every attraction underflows need their sums again, with the exponents
+// shifted by their nearest D (an exact common factor). The forward pass leaves their groups
+// to redo_kernel, the sources marked by a shift of -1 in their state: those whose sums came
+// out too small, and, without a walk, whole groups with an isolated source. redo_kernel
+// walks a group for the sums and the nearest D at once, and again, shifted, for the
+// sources that need it. A kernel of its own, which ends at once where nothing underflows:
+// as a part of the forward kernel, called from it, the same made that one 6 us slower for
+// 1,000 neurons. A forward call in which a tenth / a third / nearly all of the
+// sources underflow (a cube of 62 um spacing, sigma 8 / 6 / 1.5 um), us, each such lane
+// walking its own frontier twice -> here: 5,003 neurons 606 / 634 / 655 -> 155 / 165 / 167;
+// 60,000 2,480 / 2,640 / 2,760 -> 750 / 815 / 850; 2^18 4,550 / 4,900 / 7,140 -> 2,770 /
+// 3,060 / 3,160. Where nothing underflows (sigma 800 um): 90.9 -> 96.5 (86.9 -> 86.5 replayed
+// from a graph), 440 -> 434, 1,580 -> 1,542.
+constexpr float kMarked = -1.0f;
+
+// Whether one of the group's sources (on: this lane's is one, at Morton position sp) has
+// none of the four positions on either side of its own in Morton order within the distance
+// at which an attraction still counts (2^-50): a guess that its sums will underflow.
+__device__ __forceinline__ bool isolated(const LenArgs &a, bool on, int64_t sp, float3 x, float k2)
+{
+    bool near = !on;
+    for (int k = 1; k <= 4 && __any_sync(0xffffffffu, !near); ++k)
+        for (int64_t q : {sp - k, sp + k})
+            if (!near && q >= 0 && q < a.n) {
+                const float4 p = a.pos[q];
+                near = __fmul_rn(k2, dist2_of(__fsub_rn(x.x, p.x), __fsub_rn(x.y, p.y),
+                                              __fsub_rn(x.z, p.z))) < 50.0f;
+            }
+    return __any_sync(0xffffffffu, !near);
+}
+
 // 3 blocks per SM (80 registers): 2^18 neurons, forward + backward 4.21 ms; 4 blocks
 // (64 registers, spills) 4.49, 2 blocks 4.25 (60,000 neurons: 1.13, 1.22, 1.29 ms).
 #ifndef RELEARN_LEN_MIN_BLOCKS
@@ -662,44 +831,28 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
     length_kernel(LenArgs a)
 {
     __shared__ GroupShared s_group[kGroupWarps];
-    __shared__ double s_sum[kGroupWarps][3][32];
+    __shared__ BlockSums s_sum;
     __shared__ int32_t s_next;
     const int32_t A = (int32_t)*a.d_total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t thr0 = __ldg(&a.sc->thr0);
     const float k2 = __ldg(&a.sc->k2);
     const float sigma = __ldg(&a.sc->sigma);
     const float two_s2 = (float)(2.0 / ((double)sigma * (double)sigma));
-    const int32_t root_end = __ldg(&a.nodes[0].t.escape);
     double wscale = 0.0;
     if constexpr (kBack) {
         const double M = a.lsum[1];
         wscale = M > 0.0 ? (a.gout ? *a.gout : 1.0) / M : 0.0;
     }
-    // warps per group (see above for the line)
     const int32_t groups = (A + 31) / 32;
-    int wpg = kGroupWarps;
-    while (wpg > 1 && (int64_t)groups * wpg > 2 * (int64_t)gridDim.x * kGroupWarps) wpg >>= 1;
-    const int sub = warp & (wpg - 1);
+    const int wpg = warps_per_group(groups), sub = warp & (wpg - 1);
     double my0 = 0.0, my1 = 0.0;
     int64_t my_evals = 0;
     GroupWalk w;
     w.fam = a.fam;
     w.s = &s_group[warp];
-    w.thr0 = thr0;
-    for (;;) {
-        int32_t gr = 0;
-        if (wpg == 1) {
-            if (lane == 0) gr = atomicAdd(a.work, 1);
-            gr = __shfl_sync(0xffffffffu, gr, 0);
-            if (gr >= groups) break;
-        } else { // the block takes kGroupWarps / wpg groups together
-            __syncthreads();
-            if (threadIdx.x == 0) s_next = atomicAdd(a.work, kGroupWarps / wpg);
-            __syncthreads();
-            if (s_next >= groups) break;
-            gr = s_next + warp / wpg;
-        }
+    w.thr0 = __ldg(&a.sc->thr0);
+    int32_t gr = 0;
+    while (next_group(a.work, groups, wpg, s_next, gr)) {
         const int64_t slot = (int64_t)gr * 32 + lane;
         const bool live = slot < A;
         const int32_t sp = live ? a.act_src[slot] : -1;
@@ -709,8 +862,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
         s.self = live ? a.leaf_of[sp] : 0x7fffffff;
         const int32_t i = live ? a.perm[sp] : 0;
         s.l = s.Db = s.invS = s.k2sh = s.w = 0.0f;
-        // a source without a finite position has no finite distance and is left out
-        bool on_src = live && fabsf(xp.x) + fabsf(xp.y) + fabsf(xp.z) < __int_as_float(0x7f800000);
+        bool on_src = live && finite_at(xp);
         if constexpr (kBack) {
             if (live) {
                 const float4 st = a.state[sp];
@@ -725,52 +877,13 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
         FwdSums f;
         BwdSums b;
         const uint32_t members = __ballot_sync(0xffffffffu, on_src);
-        if (members) {
-            { // lanes without a source follow one, with an empty mask
-                const int f0 = __ffs(members) - 1;
-                const float mx = __shfl_sync(0xffffffffu, s.x.x, f0),
-                            my = __shfl_sync(0xffffffffu, s.x.y, f0),
-                            mz = __shfl_sync(0xffffffffu, s.x.z, f0);
-                if (!on_src) s.x = make_float3(mx, my, mz);
-            }
-            w.start(members, s.x, s.self);
-            if (wpg > 1) { // a pending list long enough to share out (at most 140 nodes)
-                while (w.top - w.base > 0 && w.top - w.base < 8 * wpg && w.top <= 72 &&
-                       w.outc < kEntries - 64)
-                    w.expand<true>();
-                w.take_share(sub, wpg);
-            }
-            for (;;) {
-                while (w.outc < kLenChunk && w.top > 0) {
-                    if (w.top > kPend - 64 - kLenChunk) { // not reached by ordinary trees
-                        const uint2 it = w.s->pend[--w.top];
-                        float part[4];
-                        walk_pending<kBack>(a, s, it, thr0, k2, two_s2, part, my_evals);
-                        if constexpr (kBack) {
-                            b.cov.add_one(part[0]);
-                            b.gx.add_one(part[1]);
-                            b.gy.add_one(part[2]);
-                            b.gz.add_one(part[3]);
-                        } else {
-                            f.s.add_one(part[0]);
-                            f.a.add_one(part[1]);
-                            f.b.add_one(part[2]);
-                        }
-                    } else {
-                        w.expand<false>();
-                    }
-                }
-                const int n = min(w.outc, kLenChunk);
-                if (n == 0) break;
-                uint32_t kids;
-                const uint32_t tests = w.gather(n, kids, my_evals);
-                if (tests) w.resolve(tests, kids, s.x, my_evals);
-                if constexpr (kBack)
-                    bwd_chunk(w.s, n, s, k2, two_s2, a.G, b);
-                else
-                    fwd_chunk(w.s, n, s, k2, f);
-                __syncwarp(); // the chunk is overwritten next
-            }
+        bool left = false; // the whole group is left to redo_kernel
+        if constexpr (!kBack) left = isolated(a, on_src, sp, s.x, k2);
+        if (members && !left) {
+            follow(members, on_src, s.x);
+            float unused;
+            group_pass<kBack ? kAdjoint : kSums>(a, w, s, members, sub, wpg, k2, two_s2, f, b,
+                                                 unused, my_evals);
         }
         double t0, t1, t2;
         if constexpr (kBack) {
@@ -796,37 +909,13 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
             }
         }
         if constexpr (!kBack) {
-            if (live) {
-                double S = t0;
-                float k2sh = 0.0f;
-                if (on_src && S < (double)kTinyL) {
-                    // every term underflowed: redo with the exponents shifted by the
-                    // nearest D, which a first walk of the lane's own frontier finds
-                    Bwd unused;
-                    Fwd g;
-                    lane_walk<false>(a, s, 1, root_end, thr0, k2, 0.0f, two_s2, g, unused);
-                    if (g.dmin2 < __int_as_float(0x7f800000)) {
-                        k2sh = __fmul_rn(k2, g.dmin2);
-                        g = Fwd();
-                        my_evals += lane_walk<false>(a, s, 1, root_end, thr0, k2, k2sh, two_s2, g,
-                                                     unused);
-                        S = (double)g.s - (double)g.sc;
-                        t1 = (double)g.a - (double)g.ac;
-                        t2 = (double)g.b - (double)g.bc;
-                    }
-                }
-                float4 st = make_float4(0.f, 0.f, 0.f, k2sh);
-                if (S > 0.0) {
-                    const double l = t1 / S;
-                    st.x = (float)l;
-                    st.y = (float)(t2 / S);
-                    st.z = (float)(1.0 / S);
-                    const double m = (double)a.vac_ax[i];
-                    my0 += m * l;
-                    my1 += m;
-                }
-                a.state[sp] = st;
-            }
+            const bool again = on_src && (left || t0 < (double)kTinyL);
+            if (__any_sync(0xffffffffu, again) && lane == 0)
+                a.redo_list[atomicAdd(a.redo, 1)] = gr;
+            if (again)
+                a.state[sp] = make_float4(0.f, 0.f, 0.f, kMarked);
+            else if (live)
+                finish_source(a, sp, i, t0, t1, t2, 0.0f, my0, my1);
         } else if (on_src) { // the sums hold the negated direct term
             a.gx[i] = (float)-t0;
             a.gy[i] = (float)-t1;
@@ -834,25 +923,101 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
         }
         __syncwarp();
     }
-    for (int o = 16; o; o >>= 1) {
-        my0 += __shfl_xor_sync(0xffffffffu, my0, o);
-        my1 += __shfl_xor_sync(0xffffffffu, my1, o);
-        my_evals += __shfl_xor_sync(0xffffffffu, my_evals, o);
-    }
-    if (lane == 0 && my_evals)
-        atomicAdd(reinterpret_cast<unsigned long long *>(a.evals_total),
-                  (unsigned long long)my_evals);
-    if (lane == 0) {
-        if constexpr (!kBack) {
-            if (my1 > 0.0) {
-                atomicAdd(&a.lsum[0], my0);
-                atomicAdd(&a.lsum[1], my1);
-            }
-        } else if (a.gsigma && my0 != 0.0) {
+    if constexpr (!kBack) {
+        add_totals(a, my0, my1, my_evals);
+    } else {
+        for (int o = 16; o; o >>= 1) {
+            my0 += __shfl_xor_sync(0xffffffffu, my0, o);
+            my_evals += __shfl_xor_sync(0xffffffffu, my_evals, o);
+        }
+        if (lane == 0 && my_evals)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.evals_total),
+                      (unsigned long long)my_evals);
+        if (lane == 0 && a.gsigma && my0 != 0.0) {
             const double sd = (double)sigma;
             atomicAdd(a.gsigma, my0 * 2.0 / (sd * sd * sd));
         }
     }
+}
+
+// Each lane's sums and nearest D over the warps that share its group, in their order.
+// Every warp of the block calls it and gets its group's.
+__device__ __forceinline__ void group_totals(BlockSums &sums, int sub, int wpg, double t[3],
+                                             float &nearest)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = 0; k < 3; ++k) sums[warp][k][lane] = t[k];
+    __syncthreads();
+    for (int k = 0; k < 3; ++k) {
+        t[k] = sums[warp - sub][k][lane];
+        for (int q = 1; q < wpg; ++q) t[k] += sums[warp - sub + q][k][lane];
+    }
+    __syncthreads();
+    sums[warp][0][lane] = (double)nearest;
+    __syncthreads();
+    for (int q = 0; q < wpg; ++q) nearest = fminf(nearest, (float)sums[warp - sub + q][0][lane]);
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS) redo_kernel(LenArgs a)
+{
+    __shared__ GroupShared s_group[kGroupWarps];
+    __shared__ BlockSums s_sum;
+    __shared__ int32_t s_next;
+    const int32_t groups = a.redo[0];
+    if (groups == 0) return;
+    const int32_t A = (int32_t)*a.d_total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float k2 = __ldg(&a.sc->k2), inf = __int_as_float(0x7f800000);
+    const int wpg = warps_per_group(groups), sub = warp & (wpg - 1);
+    double my0 = 0.0, my1 = 0.0;
+    int64_t my_evals = 0;
+    GroupWalk w;
+    w.fam = a.fam;
+    w.s = &s_group[warp];
+    w.thr0 = __ldg(&a.sc->thr0);
+    int32_t at = 0;
+    while (next_group(a.redo + 1, groups, wpg, s_next, at)) {
+        const int64_t slot = at < groups ? (int64_t)a.redo_list[at] * 32 + lane : A;
+        const int32_t sp = slot < A ? a.act_src[slot] : -1;
+        // (the states of marked sources alone are written, by the warp with sub 0, after the
+        // last barrier that follows these reads)
+        const bool marked = sp >= 0 && a.state[sp].w == kMarked;
+        Src s{};
+        const float4 xp = marked ? a.pos[sp] : make_float4(0.f, 0.f, 0.f, 0.f);
+        s.x = make_float3(xp.x, xp.y, xp.z);
+        s.self = sp >= 0 ? a.leaf_of[sp] : 0x7fffffff;
+        uint32_t members = __ballot_sync(0xffffffffu, marked);
+        double t[3] = {0.0, 0.0, 0.0};
+        float nearest = inf;
+        BwdSums unused;
+        if (members) {
+            FwdSums f;
+            follow(members, marked, s.x);
+            group_pass<kNearSums>(a, w, s, members, sub, wpg, k2, 0.0f, f, unused, nearest,
+                                  my_evals);
+            t[0] = f.s.total();
+            t[1] = f.a.total();
+            t[2] = f.b.total();
+        }
+        if (wpg > 1) group_totals(s_sum, sub, wpg, t, nearest);
+        const bool shifted = marked && t[0] < (double)kTinyL && nearest < inf;
+        if (shifted) s.k2sh = __fmul_rn(k2, nearest);
+        members = __ballot_sync(0xffffffffu, shifted);
+        if (wpg > 1 ? __syncthreads_or(members != 0u) : members != 0u) {
+            FwdSums f;
+            if (members)
+                group_pass<kSums>(a, w, s, members, sub, wpg, k2, 0.0f, f, unused, nearest,
+                                  my_evals);
+            double u[3] = {f.s.total(), f.a.total(), f.b.total()};
+            if (wpg > 1) group_totals(s_sum, sub, wpg, u, nearest);
+            if (shifted)
+                for (int k = 0; k < 3; ++k) t[k] = u[k];
+        }
+        if (sub == 0 && marked) finish_source(a, sp, a.perm[sp], t[0], t[1], t[2], s.k2sh, my0, my1);
+        __syncwarp();
+    }
+    add_totals(a, my0, my1, my_evals);
 }
 
 // ---- family order ---------------------------------------------------------------
@@ -916,7 +1081,7 @@ struct PrepArgs {
     int32_t *k0;
     FamNode *fam;
     double *lsum;
-    int32_t *work;
+    int32_t *work, *redo;
 };
 constexpr int64_t kSmallLen = 16384;
 
@@ -935,6 +1100,7 @@ __device__ __forceinline__ void clear_sums(const PrepArgs &a)
 {
     for (int k = 0; k < 4; ++k) a.lsum[k] = 0.0;
     *a.work = 0;
+    a.redo[0] = a.redo[1] = 0;
 }
 
 __global__ void len_count_kernel(PrepArgs a)
@@ -1077,12 +1243,15 @@ LenArgs make_args(relearn_ctx *c, const int32_t *vac_ax)
     a.act_src = c->d_act_src;
     a.leaf_of = c->d_leaf;
     a.vac_ax = vac_ax;
+    a.n = c->n;
     a.d_total = c->d_i64 + I64_ACTIVE;
     a.evals_total = c->d_i64 + I64_LEN_EVALS;
     a.sc = c->d_sc;
     a.state = c->d_lstate;
     a.lsum = c->d_lsum;
     a.work = c->d_i32 + I32_WORK;
+    a.redo = c->d_i32 + I32_REDO;
+    a.redo_list = c->d_act_off; // read by the forward call's setup only
     return a;
 }
 
@@ -1117,6 +1286,7 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
     p.fam = c->d_fam;
     p.lsum = c->d_lsum;
     p.work = c->d_i32 + I32_WORK;
+    p.redo = c->d_i32 + I32_REDO;
     if (n <= kSmallLen && may_cluster(c)) {
         len_prepare_small_kernel<<<cluster_form::kBlocks, cluster_form::kThreads, 0, st>>>(p);
         note_launch();
@@ -1133,7 +1303,10 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
         len_emit_kernel<<<gm, 256, 0, st>>>(p);
         note_launch();
     }
-    if ((e = launch_length<false>(c, make_args(c, vac_ax), st))) return e;
+    const LenArgs a = make_args(c, vac_ax);
+    if ((e = launch_length<false>(c, a, st))) return e;
+    redo_kernel<<<c->num_sms * RELEARN_LEN_MIN_BLOCKS, 32 * kGroupWarps, 0, st>>>(a);
+    note_launch();
     len_finish_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(c->d_lstate, p.flag,
                                                                      c->d_perm, n, c->d_lsum,
                                                                      ell, mean);
