@@ -40,6 +40,7 @@
 
 #include "cluster.cuh"
 #include "internal.h"
+#include "last_start.h"
 #include "scan_pair.cuh"
 
 namespace rl {
@@ -862,14 +863,7 @@ __device__ __forceinline__ int split_locate(const SplitLists &L, int n_rec, doub
 {
     const int per = (n_rec + 31) >> 5;
     const int nb = (n_rec + per - 1) / per; // non-empty blocks
-    int k = 0; // the last block that starts at or before tgt (the starts do not decrease)
-    for (int hi = nb - 1; k < hi;) {
-        const int mid = (k + hi + 1) >> 1;
-        if (L.start[mid] <= tgt)
-            k = mid;
-        else
-            hi = mid - 1;
-    }
+    const int k = last_start(L.start, nb, tgt); // the last block that starts at or before tgt
     const int q0 = k * per, q1 = min(q0 + per, n_rec);
     double run = 0.0;
     for (int q = q0; q < q1; ++q) {
