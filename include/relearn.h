@@ -72,7 +72,7 @@ typedef struct relearn_ctx relearn_ctx;
  *             0 = the default: one source per warp when the update has at most 9 sources
  *             per resident warp of the union kernel, else unions chosen per warp: its 32
  *             sources (Morton order) cut at the boundaries of the deepest cells (depth 8 at
- *             most) that make at most 8 pieces (12 in updates of few sources), one union
+ *             most) that make at most 6 pieces (12 in updates of few sources), one union
  *             per piece;
  *             1000 + 100 * d + r (d = 0..10, r = 0..10, r unused) = the default with the
  *             pieces cut at the boundaries of depth-d cells;
@@ -123,7 +123,9 @@ typedef struct {
     float ms_reduce;        /* bottom-up octree update */
     float ms_search;        /* query setup + search kernel */
     float ms_search_kernel; /* the search kernel alone */
-    float ms_accept, ms_apply, ms_total;
+    float ms_accept, ms_apply, ms_total; /* networks of at most 40,960 neurons (on a context
+                               of at most 327,680 searches and synapses) accept and apply
+                               in one launch: its time is ms_accept, ms_apply about 0 */
     int32_t reserved;
     int64_t searches_total;     /* searches of every update since the context was created */
     int64_t evals_total;        /* node evaluations (count > 0) of the searches of updates run

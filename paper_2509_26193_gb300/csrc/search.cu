@@ -74,13 +74,16 @@ constexpr float kTiny = 8.673617e-19f; // 2^-60
 // batch 9.81 / 10.09 / 10.55, slab 48.4 / 48.4 / 48.5: hence 5.
 constexpr int kMaxCutDepth = 8, kMaxCuts = 5, kMaxCutsFew = 11, kFewSources = 20;
 // The default also looks at how many sources the update has, per resident warp of
-// the union kernel (W = 9,728 on 152 SMs at 8 blocks per SM; the sweeps below were
-// taken at 6 blocks, W = 7,296, and the threshold rechecked at 8). Per-update sweeps
-// on the 2^20-neuron clustered network (ten successive updates, 907k down to 2.4k
-// sources): with at most kSplitWaves * W sources the split kernel (one warp per
-// source) wins (61.8k sources: 1.67 ms against 1.84 ms; 162k: 4.73 ms against
-// 2.46 ms), on small trees as well (4096-neuron cube, 4096 sources: 0.10 ms against
-// 0.46 ms).
+// the union kernel (W = 9,728 on 152 SMs at 8 blocks per SM): with at most kSplitWaves * W
+// = 87,552 sources the split kernel (one warp per source) runs. Successive updates, split
+// against union, ms: 2^20 clusters 160,903 sources 3.21 / 2.04, 61,113 1.11 / 1.48, 24,010
+// 0.40 / 1.23; 2^20 cube 152,558 2.80 / 1.71, 58,733 1.01 / 1.42; 200,000 in a cube 78,676
+// 1.24 / 1.23; 300,007 clustered at theta 0.2 45,834 2.48 / 2.59; 50,021 clustered 43,310
+// 0.97 / 1.47; a 4,096-neuron cube 3,526 0.06 / 0.35. The line fits networks of 2^20; in
+// smaller ones, whose sources lie denser on a smaller tree, the union kernel overtakes
+// earlier (100,000 clustered, 86,446 sources 2.96 / 1.83, 40,078 1.42 / 1.60). It decides
+// which kernel draws, whose sums round differently, so moving it changes draws that lie
+// within a rounding of a boundary.
 constexpr int kSplitWaves = 9;
 
 // A node of depth d is accepted iff d^2 > thr0 / 4^d, thr0 = (root length / theta)^2
@@ -237,7 +240,7 @@ struct SearchArgs {
     uint64_t seed;
     uint32_t step;
     int forced_group; // 0 = choose per warp; 1, 8, 16, 32 = union width; 2 = split
-    int spread_depth;  // cut depth of union pieces (-1: the default by source density)
+    int spread_depth;  // cut depth of union pieces (-1: chosen per warp, see kMaxCuts)
     int32_t split_below; // with forced_group 0: split kernel for at most this many sources
     int split_cap;       // ranges per source in the split kernel (split_capacity)
     // deferred restarts (RELEARN_FLAG_REGROUP): searches whose first draw is an inner

@@ -1,5 +1,6 @@
 // Stable LSD radix sort of (key, int32 value) pairs with 8-bit digits, one pass over the
-// data per digit: a first kernel counts the digits of every position at once; each pass
+// data per digit (the published one-sweep scheme of Adinets and Merrill 2022, on the
+// decoupled look-back of Merrill and Garland 2016): a first kernel counts the digits of every position at once; each pass
 // then takes its tiles by ticket, ranks a tile's keys (each warp with eight votes per key, the
 // warps ordered by a per-digit prefix), publishes the tile's digit counts and adds up those of
 // the tiles before it (decoupled look-back, one thread per digit), and scatters.
