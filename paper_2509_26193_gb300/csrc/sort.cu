@@ -168,10 +168,12 @@ __global__ void __launch_bounds__(kThreads)
             }
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) wcnt[w][d] += loc;
-            // the counts of the tiles before this one, the nearest eight at a time
-            uint32_t prefix = 0;
+            // the counts of the tiles before this one, the nearest eight at a time: the words
+            // themselves are added up, and what marks them is taken off at the end
+            uint32_t words = 0;
             int spin = 0;
-            for (int64_t t = tile - 1; t >= 0;) {
+            int64_t t = tile - 1;
+            while (t >= 0) {
                 uint32_t f[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     if (done || !state_published(f[q])) break; // read again
-                    prefix += state_value(f[q]);
+                    words += f[q];
                     done = state_is_prefix(f[q]);
                     --t;
                 }
@@ -192,6 +194,8 @@ __global__ void __launch_bounds__(kThreads)
                     break;
                 }
             }
+            const uint32_t prefix =
+                tile > 0 ? state_sum(words, (uint32_t)(tile - 1 - t)) : 0u;
             if (tile > 0) st[tile * kRadix + d] = state_of_prefix(prefix + cnt);
             s_base[d] = start + prefix - loc;
         }

@@ -16,9 +16,11 @@ RELEARN_HOST_DEVICE uint32_t state_of_count(uint32_t count) { return count + 1u;
 RELEARN_HOST_DEVICE uint32_t state_of_prefix(uint32_t prefix) { return kStatePrefix | prefix; }
 RELEARN_HOST_DEVICE bool state_published(uint32_t s) { return s != 0u; }
 RELEARN_HOST_DEVICE bool state_is_prefix(uint32_t s) { return (s & kStatePrefix) != 0u; }
-RELEARN_HOST_DEVICE uint32_t state_value(uint32_t s)
+// The sum held by n words read from a tile backwards, n - 1 counts and then a prefix, whose
+// sum as words is given (modulo 2^32).
+RELEARN_HOST_DEVICE uint32_t state_sum(uint32_t words, uint32_t n)
 {
-    return state_is_prefix(s) ? s & ~kStatePrefix : s - 1u;
+    return words - (n - 1u) - kStatePrefix;
 }
 
 } // namespace rl

@@ -19,13 +19,14 @@ extern "C" int published(uint32_t s) { return state_published(s); }
 // the digits before tile n: counts back to the nearest prefix; -1: not published
 extern "C" int64_t look_back(const uint32_t *state, int64_t n)
 {
-    uint32_t sum = 0;
-    for (int64_t t = n - 1; t >= 0; --t) {
+    uint32_t words = 0;
+    int64_t t = n - 1;
+    for (bool done = false; !done; --t) {
         if (!state_published(state[t])) return -1;
-        sum += state_value(state[t]);
-        if (state_is_prefix(state[t])) break;
+        words += state[t];
+        done = state_is_prefix(state[t]);
     }
-    return sum;
+    return state_sum(words, (uint32_t)(n - 1 - t));
 }
 """
 MOST = 0x7FFFFFF0  # elements a sort may be given
