@@ -154,7 +154,7 @@ struct relearn_ctx {
 enum { I64_Q = 0, I64_FAILED, I64_DECLINED, I64_FORMED, I64_NSYN, I64_BROKEN, I64_SCAN_TOTAL,
        I64_NODES, I64_Q_TOTAL, I64_EVALS_TOTAL, I64_ACTIVE, I64_STEPS_TOTAL, I64_LEN_EVALS };
 enum { I32_N = 0, I32_Q, I32_NSYN, I32_NEW, I32_NODES, I32_WORK, I32_ACTIVE, I32_RQ, I32_BASE,
-       I32_LONG, I32_REDO, I32_REDO_WORK };
+       I32_LONG, I32_REDO, I32_REDO_WORK, I32_REDO_DONE };
 
 namespace rl {
 

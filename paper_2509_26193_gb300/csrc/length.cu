@@ -51,13 +51,16 @@ struct LenArgs {
     const int32_t *__restrict__ leaf_of;
     const int32_t *__restrict__ vac_ax;
     int64_t n;              // neurons
+    const Geom *geom;       // the network's
     const int64_t *d_total; // active sources
-    int32_t *redo;          // groups left to redo_kernel: their number, its work counter
+    int32_t *redo;          // groups left to redo_kernel: their number, its work counter,
+                            // its blocks done
     int32_t *redo_list;     // [n] which
     int64_t *evals_total;   // candidates visited (both passes)
     const SearchConst *sc;
     float4 *state;  // [n] per Morton position
     double *lsum;   // [4]
+    double *mean;   // forward: the caller's, or NULL
     int32_t *work;
     // backward
     double *G;           // [4 * nodes] centroid adjoints (x, y, z, unused) in FP64
@@ -798,14 +801,14 @@ __device__ __forceinline__ void add_totals(const LenArgs &a, double my0, double 
 // to redo_kernel, the sources marked by a shift of -1 in their state: those whose sums came
 // out too small, and, without a walk, whole groups with an isolated source. redo_kernel
 // walks a group for the sums and the nearest D at once, and again, shifted, for the
-// sources that need it. A kernel of its own, which ends at once where nothing underflows:
-// as a part of the forward kernel, called from it, the same made that one 6 us slower for
-// 1,000 neurons. A forward call in which a tenth / a third / nearly all of the
-// sources underflow (a cube of 62 um spacing, sigma 8 / 6 / 1.5 um), us, each such lane
-// walking its own frontier twice -> here: 5,003 neurons 606 / 634 / 655 -> 155 / 165 / 167;
-// 60,000 2,480 / 2,640 / 2,760 -> 750 / 815 / 850; 2^18 4,550 / 4,900 / 7,140 -> 2,770 /
-// 3,060 / 3,160. Where nothing underflows (sigma 800 um): 90.9 -> 96.5 (86.9 -> 86.5 replayed
-// from a graph), 440 -> 434, 1,580 -> 1,542.
+// sources that need it. It also forms the mean, which is all it does where nothing
+// underflows. A kernel of its own: as a part of the forward kernel, called from it, the
+// same made that one 6 us slower for 1,000 neurons. A forward call in which a tenth / a
+// third / nearly all of the sources underflow (a cube of 62 um spacing, sigma 8 / 6 / 1.5
+// um), us, each such lane walking its own frontier twice -> here: 5,003 neurons 606 / 634 /
+// 655 -> 130 / 135 / 138; 60,000 2,480 / 2,640 / 2,760 -> 747 / 812 / 840; 2^18 4,550 / 4,900 /
+// 7,140 -> 2,775 / 3,060 / 3,155. Where nothing underflows (sigma 800 um, replayed from a
+// graph): 86 -> 84, 419 -> 407, 1,560 -> 1,510; called directly 91 -> 96 (5,003 neurons).
 constexpr float kMarked = -1.0f;
 
 // Whether one of the group's sources (on: this lane's is one, at Morton position sp) has
@@ -854,6 +857,9 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
     w.fam = a.fam;
     w.s = &s_group[warp];
     w.thr0 = __ldg(&a.sc->thr0);
+    // in a domain whose diagonal is within an attraction's reach no source is isolated
+    const float ext = kBack ? 0.0f : (float)a.geom->ext;
+    const bool wide = 3.0f * k2 * ext * ext > 50.0f;
     int32_t gr = 0;
     while (next_group(a.work, groups, wpg, s_next, gr)) {
         const int64_t slot = (int64_t)gr * 32 + lane;
@@ -881,7 +887,8 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS)
         BwdSums b;
         const uint32_t members = __ballot_sync(0xffffffffu, on_src);
         bool left = false; // the whole group is left to redo_kernel
-        if constexpr (!kBack) left = isolated(a, on_src, sp, s.x, k2);
+        if constexpr (!kBack)
+            if (wide) left = isolated(a, on_src, sp, s.x, k2);
         if (members && !left) {
             follow(members, on_src, s.x);
             float unused;
@@ -962,13 +969,26 @@ __device__ __forceinline__ void group_totals(BlockSums &sums, int sub, int wpg, 
     __syncthreads();
 }
 
+// mean = sum m l / M (NaN when M = 0).
+__device__ __forceinline__ void publish_mean(const LenArgs &a)
+{
+    const volatile double *sum = a.lsum;
+    const double M = sum[1];
+    const double m = M > 0.0 ? sum[0] / M : __longlong_as_double(0x7ff8000000000000LL);
+    a.lsum[2] = m;
+    if (a.mean) *a.mean = m;
+}
+
 __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS) redo_kernel(LenArgs a)
 {
     __shared__ GroupShared s_group[kGroupWarps];
     __shared__ BlockSums s_sum;
     __shared__ int32_t s_next;
     const int32_t groups = a.redo[0];
-    if (groups == 0) return;
+    if (groups == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) publish_mean(a);
+        return;
+    }
     const int32_t A = (int32_t)*a.d_total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const float k2 = __ldg(&a.sc->k2), inf = __int_as_float(0x7f800000);
@@ -1017,10 +1037,17 @@ __global__ void __launch_bounds__(32 * kGroupWarps, RELEARN_LEN_MIN_BLOCKS) redo
             if (shifted)
                 for (int k = 0; k < 3; ++k) t[k] = u[k];
         }
-        if (sub == 0 && marked) finish_source(a, sp, a.perm[sp], t[0], t[1], t[2], s.k2sh, my0, my1);
+        if (sub == 0 && marked)
+            finish_source(a, sp, a.perm[sp], t[0], t[1], t[2], s.k2sh, my0, my1);
         __syncwarp();
     }
     add_totals(a, my0, my1, my_evals);
+    __threadfence(); // the totals, before the block counts as done
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.redo + 2, 1) == (int32_t)gridDim.x - 1) {
+        __threadfence();
+        publish_mean(a);
+    }
 }
 
 // ---- family order ---------------------------------------------------------------
@@ -1103,7 +1130,7 @@ __device__ __forceinline__ void clear_sums(const PrepArgs &a)
 {
     for (int k = 0; k < 4; ++k) a.lsum[k] = 0.0;
     *a.work = 0;
-    a.redo[0] = a.redo[1] = 0;
+    a.redo[0] = a.redo[1] = a.redo[2] = 0;
 }
 
 __global__ void len_count_kernel(PrepArgs a)
@@ -1149,20 +1176,13 @@ __global__ void __cluster_dims__(cluster_form::kBlocks, 1, 1)
     CLUSTER_STRIDE(v, m) family_emit(a.nodes, a.parent, (int32_t)v, a.k0, a.fam);
 }
 
-// mean = sum m l / M (NaN when M = 0); ell[id] = l (NaN for excluded neurons).
+// ell[id] = l (NaN for excluded neurons).
 __global__ void len_finish_kernel(const float4 *__restrict__ state,
                                   const int32_t *__restrict__ flag,
-                                  const int32_t *__restrict__ perm, int64_t n, double *lsum,
-                                  float *ell, double *mean)
+                                  const int32_t *__restrict__ perm, int64_t n, float *ell)
 {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid == 0) {
-        const double m = lsum[1] > 0.0 ? lsum[0] / lsum[1] : __longlong_as_double(0x7ff8000000000000LL);
-        lsum[2] = m;
-        if (mean) *mean = m;
-    }
-    if (!ell) return;
-    for (int64_t s = tid; s < n; s += (int64_t)gridDim.x * blockDim.x) {
+    GRID_STRIDE(s, n)
+    {
         const float4 st = state[s];
         ell[perm[s]] = flag[s] && st.z > 0.0f ? st.x : __int_as_float(0x7fc00000);
     }
@@ -1247,6 +1267,7 @@ LenArgs make_args(relearn_ctx *c, const int32_t *vac_ax)
     a.leaf_of = c->d_leaf;
     a.vac_ax = vac_ax;
     a.n = c->n;
+    a.geom = c->d_geom;
     a.d_total = c->d_i64 + I64_ACTIVE;
     a.evals_total = c->d_i64 + I64_LEN_EVALS;
     a.sc = c->d_sc;
@@ -1306,14 +1327,18 @@ cudaError_t length_forward(relearn_ctx *c, const int32_t *vac_ax, float *ell, do
         len_emit_kernel<<<gm, 256, 0, st>>>(p);
         note_launch();
     }
-    const LenArgs a = make_args(c, vac_ax);
+    LenArgs a = make_args(c, vac_ax);
+    a.mean = mean;
     if ((e = launch_length<false>(c, a, st))) return e;
-    redo_kernel<<<c->num_sms * RELEARN_LEN_MIN_BLOCKS, 32 * kGroupWarps, 0, st>>>(a);
+    // at most a block per group (every block shares one group among its warps then)
+    const int64_t most = std::min<int64_t>((n + 31) / 32, c->num_sms * RELEARN_LEN_MIN_BLOCKS);
+    redo_kernel<<<(unsigned)most, 32 * kGroupWarps, 0, st>>>(a);
     note_launch();
-    len_finish_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(c->d_lstate, p.flag,
-                                                                     c->d_perm, n, c->d_lsum,
-                                                                     ell, mean);
-    note_launch();
+    if (ell) {
+        len_finish_kernel<<<grid_for(n, 256, c->num_sms), 256, 0, st>>>(
+            c->d_lstate, p.flag, c->d_perm, n, ell);
+        note_launch();
+    }
     return cudaGetLastError();
 }
 
